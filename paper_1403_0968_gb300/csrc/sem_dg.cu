@@ -3,13 +3,8 @@
 // Per element and node the kernel forms the fluxes F, G of the conservative shallow-water system
 // from the nodal fields, combines them with the element's affine-map factors into
 // Xr = rx F + ry G and Xs = sx F + sy G, and applies the weak derivative matrices:
-// rhs = Drw Xr + Dsw Xs + S.  A block of 256 threads takes batches of floor(256 / Np) elements,
-// one thread per element node, and stays resident over many batches (one block per free slot of
-// the device), so that it loads the operators once; the two Np x Np operators (rows zero padded to an odd number of 16-byte
-// vectors, so that threads on consecutive rows hit distinct banks) and the block's Xr, Xs sit in
-// shared memory and are read 16 bytes at a time; every thread of an element reads the same X
-// vector (a broadcast).  Per element the kernel reads 5 Np field
-// values and 4 factors and writes 3 Np values; it performs 12 Np^2 flops in the products.
+// rhs = Drw Xr + Dsw Xs + S.  Per element it reads 5 Np field values and 4 factors, writes 3 Np values
+// and performs 12 Np^2 flops in the products (k_dg_volume has the layout and its reasons).
 //
 // The operators are built on the host in FP64 from the orthonormal (Dubiner) basis of the
 // triangle: psi_ij = P_i(a) ((1-s)/2)^i P_j^(2i+1,0)(s) / sqrt(2 / ((2i+1)(i+j+1))) with the
@@ -21,26 +16,20 @@
 
 #include "../../include/sem_dg.h"
 #include "sem_internal.h"
+#include "sem_tma.cuh"
 
 __device__ int g_dg_bad;  // zero-area / clockwise triangle flag of sem_dg_geometry
 
 namespace {
 
-constexpr int DG_NT = 256;
-
 __host__ __device__ constexpr int dg_np(int N) { return (N + 1) * (N + 2) / 2; }
-// Row stride of the operators and of the X rows in shared memory, in elements of a type of `es`
-// bytes: a whole number of 16-byte vectors (zero padded), and an odd number of them so that the
-// 16-byte row loads of eight consecutive rows fall in distinct bank groups.
+// Row stride of the operator block in device memory, in elements of a type of `es` bytes: an odd
+// number of 16-byte vectors, zero padded.
 __host__ __device__ constexpr int dg_vw(int es) { return 16 / es; }
 __host__ __device__ constexpr int dg_ld(int N, int es) {
   return ((dg_np(N) + dg_vw(es) - 1) / dg_vw(es)) % 2 ? (dg_np(N) + dg_vw(es) - 1) / dg_vw(es) * dg_vw(es)
                                                         : ((dg_np(N) + dg_vw(es) - 1) / dg_vw(es) + 1) * dg_vw(es);
 }
-__host__ __device__ constexpr int dg_xw(int N, int es) {  // X row length: Np rounded up to whole vectors
-  return (dg_np(N) + dg_vw(es) - 1) / dg_vw(es) * dg_vw(es);
-}
-
 // ---------------------------------------------------------------------------------------------
 // host: operators
 // ---------------------------------------------------------------------------------------------
@@ -150,103 +139,213 @@ void vandermonde(int N, std::vector<double> &V, std::vector<double> &Vr, std::ve
 // device: volume kernel
 // ---------------------------------------------------------------------------------------------
 
-template <typename T>
-struct alignas(16) DgVec {
-  T v[16 / sizeof(T)];
+// Layout of the volume kernel.  The products are a GEMM with M = Np rows, K = 2 Np and three columns
+// (the fields) per element.  A lane owns one element and RI of its rows (RS lanes share an element):
+// it walks the nodes once, with the six flux combinations of a node in registers (nothing of X goes
+// through shared memory), and adds their products with a column of Drw and of Dsw to 3 RI
+// accumulators.  The operator columns come from shared memory 16 bytes at a time, one load for 3 x 4
+// products; FP32 products run two rows to an instruction (FFMA2: the scalar FMA rate at half the
+// issue slots).  A warp stages the fields of its WE elements by asynchronous copies, one batch ahead,
+// and its results leave through the same buffer; warps are independent of one another.
+// What bounds it at N = 7, FP32: the operator loads (each returns 512 bytes to registers, four
+// cycles of the SM's shared-memory path, for 12 FMA cycles per scheduler) and the FMA pipe, half
+// busy; with the products left out the copies alone take 48 us of the 99 us.  212,800 triangles,
+// before (one thread per node of 1 to 3 elements, X in shared memory) / now, L2 flushed: FP32
+// N = 1..8 13 / 11, 23 / 16, 35 / 21, 81 / 33, 130 / 48, 111 / 74, 163 / 99, 326 / 150 us, FP64 N = 4
+// 1012 / 691, 8 8697 / 5199 us (the FP64 pipe: 4640 us for the products alone).
+template <typename T, int N, int RS_>
+struct DgCfg {
+  static constexpr int NP = dg_np(N), VW = dg_vw(sizeof(T)), RS = RS_;
+  static constexpr int WE = 32 / RS;                        // elements per warp
+  static constexpr int RW = sizeof(T) == 4 ? 2 : 1;         // rows per product instruction
+  static constexpr int RI = ((NP + RS - 1) / RS + RW - 1) / RW * RW;  // rows per lane
+  static constexpr int RP = (RI + VW - 1) / VW * VW;        // row stride of an operator column
+  static constexpr int QW = WE * 3 * NP, BW = WE * 2 * NP;  // field and bathymetry values of a batch
+  static constexpr int PW = 2 * QW + BW;                    // values staged per warp (fields twice)
+  static constexpr int DW = NP * RS * 2 * RP;               // operator values per block
+  static constexpr int FIT = (int)((227 * 1024 / sizeof(T) - DW) / PW);
+  // at most two warps per scheduler; a fifth alone would leave three schedulers with one each
+  static constexpr int W = FIT >= 8 ? 8 : FIT == 5 ? 4 : FIT;  // warps per block
+  static constexpr size_t SMEM = (size_t)(DW + W * PW) * sizeof(T);
+  static_assert(W >= 1 && SMEM <= 227 * 1024, "shared memory of a block");
+  static_assert(QW * sizeof(T) % 16 == 0 && BW * sizeof(T) % 16 == 0 && DW * sizeof(T) % 16 == 0, "16-byte regions");
 };
 
-// Elements per thread: with ET > 1 every operator vector a thread loads serves ET elements (fewer
-// shared-memory wavefronts per output); FP64 keeps 1 (its FMA pipe is the bound, and its shared
-// memory would not fit).  Measured on 212,800 triangles: ET = 2 1.2x over 1 at N = 6..8, slower at
-// N = 2; ET = 3 (73 registers, 3 blocks per SM) a further 5% at N = 7 and 8.5% at N = 8, level at
-// N = 6; ET = 4 (90 registers) slower.
-__host__ __device__ constexpr int dg_et(int N, int es) { return es == 4 && N >= 7 ? 3 : es == 4 && N >= 3 ? 2 : 1; }
+template <typename T, int V>
+struct alignas(V * sizeof(T)) DgVec {
+  T v[V];
+};
 
-template <typename T, int N>
-__global__ void __launch_bounds__(DG_NT) k_dg_volume(int64_t E, T g, const T *__restrict__ ops,
-                                                     const T *__restrict__ Q, const T *__restrict__ Bxy,
-                                                     const T *__restrict__ geo, T *__restrict__ rhs) {
-  constexpr int NP = dg_np(N), LD = dg_ld(N, sizeof(T)), XW = dg_xw(N, sizeof(T));
-  constexpr int ET = dg_et(N, sizeof(T)), EG = DG_NT / NP, EB = EG * ET;  // groups, elements per batch
-  constexpr int VW = dg_vw(sizeof(T)), NV = XW / VW;  // 16-byte vectors per row
-  __shared__ alignas(16) T sD[2 * NP * LD];
-  __shared__ alignas(16) T sX[EB][6][XW];
-  const int tid = threadIdx.x;
-  for (int q = tid; q < 2 * NP * LD; q += DG_NT) sD[q] = ops[q];
-  // zero the padding of the X rows (it meets the zero padding of the operator rows)
-  for (int q = tid; q < EB * 6 * (XW - NP); q += DG_NT) {
-    const int row = q / (XW - NP);
-    sX[row / 6][row % 6][NP + q % (XW - NP)] = T(0);
+// acc += operator rows times one flux value (two rows to an instruction in FP32)
+__device__ __forceinline__ void dg_fma(float *a, const float *d, float x) {
+  const float2 r = __ffma2_rn(make_float2(d[0], d[1]), make_float2(x, x), make_float2(a[0], a[1]));
+  a[0] = r.x, a[1] = r.y;
+}
+__device__ __forceinline__ void dg_fma(double *a, const double *d, double x) { *a = fma(*d, x, *a); }
+
+// 1 / h by one Newton step on the hardware's approximation (within a unit in the last place of the
+// correctly rounded value), without the branch of a full division, which would keep the fluxes of
+// the next node apart from the products of this one; the approximation itself is kept where the
+// step has no meaning (h zero or infinite)
+__device__ __forceinline__ float dg_reciprocal(float h) {
+  float r;
+  asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(h));
+  const float e = fmaf(-h, r, 1.f);
+  return e == e ? fmaf(r, e, r) : r;
+}
+__device__ __forceinline__ double dg_reciprocal(double h) { return 1.0 / h; }
+
+// n values from global to shared by the lanes of a warp, 16 bytes at a time when src starts on a
+// 16-byte boundary (wide), else one value at a time
+template <typename T>
+__device__ __forceinline__ void dg_fetch(T *dst, const T *src, int n, bool wide, int lane) {
+  constexpr int VW = dg_vw(sizeof(T));
+  int done = 0;
+  if (wide) {
+    const int nv = n / VW;
+    for (int q = lane; q < nv; q += 32)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst + q * VW)), "l"(src + q * VW) : "memory");
+    done = nv * VW;
   }
-  const int el = tid / NP, i = tid - el * NP;  // group (ET consecutive elements of a batch), node
-  const bool grp = el < EG;
-  const DgVec<T> *dr = reinterpret_cast<const DgVec<T> *>(sD + i * LD);
-  const DgVec<T> *ds = reinterpret_cast<const DgVec<T> *>(sD + NP * LD + i * LD);
-  const DgVec<T> *x0 = reinterpret_cast<const DgVec<T> *>(&sX[grp ? el * ET : 0][0][0]);
-  constexpr int XS = 6 * NV;  // vectors per element in sX
-  // persistent blocks: the operators are loaded once per block, batches of EB elements follow
-  const int64_t nbatch = (E + EB - 1) / EB;
-  for (int64_t batch = blockIdx.x; batch < nbatch; batch += gridDim.x) {
-    const int64_t e0 = batch * EB + (int64_t)el * ET;
-    T h[ET], bx[ET], by[ET];
-#pragma unroll
-    for (int t = 0; t < ET; ++t) {
-      const int64_t e = e0 + t;
-      h[t] = T(1), bx[t] = T(0), by[t] = T(0);
-      if (grp && e < E) {
-        const T *q = Q + e * 3 * NP + i;
-        h[t] = q[0];
-        const T hu = q[NP], hv = q[2 * NP];
-        bx[t] = Bxy[e * 2 * NP + i];
-        by[t] = Bxy[e * 2 * NP + NP + i];
-        const T rx = geo[e * 4 + 0], ry = geo[e * 4 + 1], sx = geo[e * 4 + 2], sy = geo[e * 4 + 3];
-        const T ih = T(1) / h[t], u = hu * ih, v = hv * ih, p = T(0.5) * g * h[t] * h[t];
-        const T F0 = hu, F1 = hu * u + p, F2 = hu * v;
-        const T G0 = hv, G1 = hv * u, G2 = hv * v + p;
-        T(*X)[XW] = sX[el * ET + t];
-        X[0][i] = rx * F0 + ry * G0;
-        X[1][i] = rx * F1 + ry * G1;
-        X[2][i] = rx * F2 + ry * G2;
-        X[3][i] = sx * F0 + sy * G0;
-        X[4][i] = sx * F1 + sy * G1;
-        X[5][i] = sx * F2 + sy * G2;
-      }
+  for (int q = done + lane; q < n; q += 32)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_addr(dst + q)), "l"(src + q), "n"((int)sizeof(T))
+                 : "memory");
+}
+
+template <typename T, int N, int RS_>
+__global__ void __launch_bounds__(32 * DgCfg<T, N, RS_>::W)
+    k_dg_volume(int64_t E, T g, const T *__restrict__ ops, const T *__restrict__ Q, const T *__restrict__ Bxy,
+                const T *__restrict__ geo, T *__restrict__ rhs, int wide) {
+  using C = DgCfg<T, N, RS_>;
+  constexpr int NP = C::NP, RS = C::RS, WE = C::WE, RI = C::RI, RP = C::RP, VW = C::VW, W = C::W;
+  constexpr int LD = dg_ld(N, sizeof(T));
+  extern __shared__ __align__(16) unsigned char dg_smem[];
+  T *sD = reinterpret_cast<T *>(dg_smem);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  T *sB = sD + C::DW + warp * C::PW, *sQ = sB + C::BW, *sQn = sQ + C::QW;
+  const int el = lane % WE, part = lane / WE, i0 = part * RI;
+  // a warp's batches of WE elements: consecutive ones go to different blocks, so that a mesh with
+  // fewer batches than warps spreads over the SMs
+  const int64_t nbatch = (E + WE - 1) / WE, stride = (int64_t)gridDim.x * W;
+  int64_t batch = (int64_t)warp * gridDim.x + blockIdx.x;
+  auto fetch = [&](T *dst, const T *src, int64_t b, int per, bool w) {
+    if (b < nbatch) {
+      const int64_t e0 = b * WE;
+      dg_fetch<T>(dst, src + e0 * per, (int)(E - e0 < WE ? E - e0 : WE) * per, w, lane);
     }
-    __syncthreads();
-    if (grp && e0 < E) {
-      // 16-byte loads: one operator vector serves three fields of ET elements; each X vector is the
-      // same for every thread of the element (a broadcast)
-      T a[ET][3];
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  fetch(sQ, Q, batch, 3 * NP, wide & 1);
+  // operators as [node j][row part][Drw, Dsw][rows of the part], zero padded
+  for (int q = tid; q < C::DW; q += 32 * W) {
+    const int i = q % RP, m = q / RP % 2, p = q / (2 * RP) % RS, j = q / (2 * RP * RS), row = p * RI + i;
+    sD[q] = (i < RI && row < NP) ? ops[m * NP * LD + row * LD + j] : T(0);
+  }
+  __syncthreads();
+  for (; batch < nbatch; batch += stride) {
+    const int64_t e0 = batch * WE;
+    const int ne = (int)(E - e0 < WE ? E - e0 : WE);
+    const bool live = el < ne;  // slots past the mesh work on the batch's first element and write nothing
+    const int slot = live ? el : 0;
+    const T *ge = geo + (e0 + slot) * 4, *be = sB + slot * 2 * NP;
+    T *qe = sQ + slot * 3 * NP;
+    const T rx = ge[0], ry = ge[1], sx = ge[2], sy = ge[3];
+    // the batch's fields were asked for one batch ago; its bathymetry and the next batch's fields
+    // arrive while the products run
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncwarp();
+    fetch(sB, Bxy, batch, 2 * NP, wide & 2);
+    fetch(sQn, Q, batch + stride, 3 * NP, wide & 1);
+    T acc[3][RI] = {};
+    // The RS lanes of an element take the fluxes of RS nodes, one node each, and pass them on to one
+    // another; they are formed one group of nodes ahead, beside the products of the group before.
+    auto flux = [&](int j, T(&x)[6]) {
+      const int jc = j < NP ? j : NP - 1;
+      const T h = qe[jc], hu = qe[NP + jc], hv = qe[2 * NP + jc];
+      const T ih = dg_reciprocal(h), a = hu * ih, b = hv * ih, p = T(0.5) * g * h * h;
+      const T F1 = hu * a + p, F2 = hu * b, G1 = hv * a, G2 = hv * b + p;
+      x[0] = rx * hu + ry * hv, x[1] = rx * F1 + ry * G1, x[2] = rx * F2 + ry * G2;
+      x[3] = sx * hu + sy * hv, x[4] = sx * F1 + sy * G1, x[5] = sx * F2 + sy * G2;
+      if (NP % RS != 0 && j >= NP) {  // past the last node: its products add nothing
 #pragma unroll
-      for (int t = 0; t < ET; ++t) a[t][0] = a[t][1] = a[t][2] = T(0);
+        for (int f = 0; f < 6; ++f) x[f] = T(0);
+      }
+    };
+    T x[6], xn[6];
+    flux(part, x);
+#pragma unroll 1
+    for (int j0 = 0; j0 < NP; j0 += RS) {
+      flux(j0 + RS + part, xn);
 #pragma unroll
-      for (int jv = 0; jv < NV; ++jv) {
-        const DgVec<T> wr = dr[jv], ws = ds[jv];
+      for (int k = 0; k < RS; ++k) {  // node j0 + (part ^ k), from the lane that owns it
+        T y[6];
 #pragma unroll
-        for (int t = 0; t < ET; ++t) {
-          const DgVec<T> *xt = x0 + t * XS;
-          const DgVec<T> r0 = xt[0 * NV + jv], r1 = xt[1 * NV + jv], r2 = xt[2 * NV + jv];
-          const DgVec<T> s0 = xt[3 * NV + jv], s1 = xt[4 * NV + jv], s2 = xt[5 * NV + jv];
+        for (int f = 0; f < 6; ++f) y[f] = k == 0 ? x[f] : __shfl_xor_sync(0xffffffffu, x[f], k * WE);
+        const int jk = j0 + (part ^ k), jc = NP % RS == 0 || jk < NP ? jk : NP - 1;
+        const DgVec<T, VW> *d = reinterpret_cast<const DgVec<T, VW> *>(sD + (jc * RS + part) * 2 * RP);
 #pragma unroll
-          for (int k = 0; k < VW; ++k) {
-            a[t][0] += wr.v[k] * r0.v[k] + ws.v[k] * s0.v[k];
-            a[t][1] += wr.v[k] * r1.v[k] + ws.v[k] * s1.v[k];
-            a[t][2] += wr.v[k] * r2.v[k] + ws.v[k] * s2.v[k];
+        for (int q = 0; q < RP / VW; ++q) {
+#pragma unroll
+          for (int m = 0; m < 2; ++m) {  // Drw with Xr, then Dsw with Xs
+            const DgVec<T, VW> w = d[m * (RP / VW) + q];
+#pragma unroll
+            for (int i = 0; i < VW; i += C::RW)
+              if (q * VW + i < RI) {
+#pragma unroll
+                for (int f = 0; f < 3; ++f) dg_fma(&acc[f][q * VW + i], &w.v[i], y[3 * m + f]);
+              }
           }
         }
       }
 #pragma unroll
-      for (int t = 0; t < ET; ++t) {
-        const int64_t e = e0 + t;
-        if (e < E) {
-          T *o = rhs + e * 3 * NP + i;
-          o[0] = a[t][0];
-          o[NP] = a[t][1] - g * h[t] * bx[t];
-          o[2 * NP] = a[t][2] - g * h[t] * by[t];
+      for (int f = 0; f < 6; ++f) x[f] = xn[f];
+    }
+    // bathymetry source at this lane's rows, then the results take the place of the fields
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncwarp();
+    // (rows in pairs where every row of pairs starts on one)
+    constexpr int VE = NP % 2 == 0 && RI % 2 == 0 ? 2 : 1;
+    using VR = DgVec<T, VE>;
+    VR *q0 = reinterpret_cast<VR *>(qe + i0);
+    const VR *b0 = reinterpret_cast<const VR *>(be + i0);
+#pragma unroll
+    for (int r = 0; r < RI / VE; ++r)
+      if (i0 + r * VE < NP) {
+        const VR h = q0[r], bx = b0[r], by = b0[NP / VE + r];
+#pragma unroll
+        for (int k = 0; k < VE; ++k) {
+          acc[1][r * VE + k] -= g * h.v[k] * bx.v[k];
+          acc[2][r * VE + k] -= g * h.v[k] * by.v[k];
         }
       }
+    __syncwarp();
+    if (live) {
+#pragma unroll
+      for (int r = 0; r < RI / VE; ++r)
+        if (i0 + r * VE < NP) {
+#pragma unroll
+          for (int f = 0; f < 3; ++f) {
+            VR o;
+#pragma unroll
+            for (int k = 0; k < VE; ++k) o.v[k] = acc[f][r * VE + k];
+            q0[f * (NP / VE) + r] = o;
+          }
+        }
     }
-    __syncthreads();  // the next batch overwrites sX
+    __syncwarp();
+    T *out = rhs + e0 * 3 * NP;
+    const int n = ne * 3 * NP;
+    int done = 0;
+    if (wide & 4) {
+      using VO = DgVec<T, VW>;
+      for (int q = lane; q < n / VW; q += 32) reinterpret_cast<VO *>(out)[q] = reinterpret_cast<const VO *>(sQ)[q];
+      done = n / VW * VW;
+    }
+    for (int q = done + lane; q < n; q += 32) out[q] = sQ[q];
+    __syncwarp();
+    T *t = sQ;
+    sQ = sQn;
+    sQn = t;
   }
 }
 
@@ -267,23 +366,40 @@ __global__ void k_dg_geometry(int64_t E, const double *__restrict__ v, T *__rest
   geo[e * 4 + 3] = (T)(xr / J);
 }
 
+template <typename T, int N, int RS>
+sem_status launch_dg_rs(int64_t E, double g, const void *ops, const void *Q, const void *Bxy, const void *geo,
+                        void *rhs, int sms, cudaStream_t s) {
+  using C = DgCfg<T, N, RS>;
+  static std::atomic<unsigned long long> attr_done;
+  SEM_CUDA_TRY((set_smem_limit_once(k_dg_volume<T, N, RS>, C::SMEM, attr_done)));
+  // persistent grid: as many blocks as fit on the device at once (each loads the operators once)
+  int per_sm = 0;
+  SEM_CUDA_TRY((cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_dg_volume<T, N, RS>, 32 * C::W, C::SMEM)));
+  const int64_t batches = (E + C::WE - 1) / C::WE, resident = (int64_t)sms * (per_sm > 0 ? per_sm : 1);
+  const int64_t blocks = batches < resident ? batches : resident;
+  auto aligned = [](const void *p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; };
+  const int wide = (aligned(Q) ? 1 : 0) | (aligned(Bxy) ? 2 : 0) | (aligned(rhs) ? 4 : 0);
+  k_dg_volume<T, N, RS><<<(unsigned)blocks, 32 * C::W, C::SMEM, s>>>(
+      E, (T)g, static_cast<const T *>(ops), static_cast<const T *>(Q), static_cast<const T *>(Bxy),
+      static_cast<const T *>(geo), static_cast<T *>(rhs), wide);
+  SEM_CUDA_TRY(cudaGetLastError());
+  return SEM_OK;
+}
+
+// Lanes per element on a mesh that fills the device: one while 3 Np accumulators fit in registers
+// beside the rest (measured at 212,800 triangles, FP32, 1 / 2 / 4 lanes: N = 4 32 / 38 / 36 us,
+// 5 48 / 52 / 56, 6 79 / 70 / 79, 7 107 / 99 / 99; FP64, 1 / 2 lanes: N = 4 674 / 855, 5 1340 / 1424).
+// Below four warps per SM, four lanes: a few elements then spread over more schedulers (FP64, 4000
+// triangles, 1 or 2 / 4 lanes: N = 3 37 / 17 us, 8 265 / 137).
 template <typename T, int N>
 sem_status launch_dg(int64_t E, double g, const void *ops, const void *Q, const void *Bxy, const void *geo,
                      void *rhs, cudaStream_t s) {
-  constexpr int EB = DG_NT / dg_np(N) * dg_et(N, sizeof(T));
-  const int64_t batches = (E + EB - 1) / EB;
-  // persistent grid: as many blocks as fit on the device at once (each loads the operators once)
-  int dev = 0, sms = 0, per_sm = 0;
+  constexpr int RS = N >= 6 ? 2 : 1;
+  int dev = 0, sms = 0;
   SEM_CUDA_TRY(cudaGetDevice(&dev));
   SEM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  SEM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_dg_volume<T, N>, DG_NT, 0));
-  const int64_t resident = (int64_t)sms * (per_sm > 0 ? per_sm : 1);
-  const int64_t blocks = batches < resident ? batches : resident;
-  k_dg_volume<T, N><<<(unsigned)blocks, DG_NT, 0, s>>>(
-      E, (T)g, static_cast<const T *>(ops), static_cast<const T *>(Q), static_cast<const T *>(Bxy),
-      static_cast<const T *>(geo), static_cast<T *>(rhs));
-  SEM_CUDA_TRY(cudaGetLastError());
-  return SEM_OK;
+  if (E < (int64_t)sms * 4 * (32 / RS)) return launch_dg_rs<T, N, 4>(E, g, ops, Q, Bxy, geo, rhs, sms, s);
+  return launch_dg_rs<T, N, RS>(E, g, ops, Q, Bxy, geo, rhs, sms, s);
 }
 
 template <typename T>
