@@ -167,6 +167,33 @@ __device__ __forceinline__ float2 dpm(float2 va, float2 vb, bool minus) {
   return make_float2(t, __fadd_rn(__fadd_rn(va.y, by), err));
 }
 
+// ---- the same operations on two independent values at once (packed FP32, f32x2) ----
+// Two FP32 operations per instruction at the scalar rate per lane: the packed forms halve the issue
+// slots and round exactly as the scalar ones.
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, neg2(b)); }
+
+// (s, c) = (dh + dl) * (vh + vl) for both halves
+__device__ __forceinline__ void dacc2_first(float2 &s, float2 &c, float2 dh, float2 dl, float2 vh, float2 vl) {
+  s = __fmul2_rn(dh, vh);
+  float2 e = __ffma2_rn(dh, vh, neg2(s));
+  e = __ffma2_rn(dh, vl, e);
+  c = __ffma2_rn(dl, vh, e);
+}
+
+// (s, c) += (dh + dl) * (vh + vl)
+__device__ __forceinline__ void dacc2(float2 &s, float2 &c, float2 dh, float2 dl, float2 vh, float2 vl) {
+  const float2 p = __fmul2_rn(dh, vh);
+  float2 e = __ffma2_rn(dh, vh, neg2(p));
+  e = __ffma2_rn(dh, vl, e);
+  e = __ffma2_rn(dl, vh, e);
+  const float2 t = __fadd2_rn(s, p);  // TwoSum(s, p)
+  const float2 z = sub2(t, s);
+  const float2 err = __fadd2_rn(sub2(s, sub2(t, z)), sub2(p, z));
+  s = t;
+  c = __fadd2_rn(c, __fadd2_rn(err, e));
+}
+
 template <int NP>
 struct DPair {
   float hi[NP * NP], lo[NP * NP];  // D[i][m] at i * NP + m
@@ -180,8 +207,8 @@ struct DPair {
 template <int NP>
 struct EvenOdd {
   static constexpr int H = NP / 2 > 0 ? NP / 2 : 1;
-  float aph[H * H], apl[H * H], amh[H * H], aml[H * H];  // forward (M = D)
-  float bph[H * H], bpl[H * H], bmh[H * H], bml[H * H];  // transposed (M = D^T)
+  // pairs (A+, A-)[i][m] at i * H + m, high and low words, for M = D (index 0) and M = D^T (index 1)
+  float2 hi[2][H * H], lo[2][H * H];
 };
 
 template <int NP>
@@ -207,126 +234,139 @@ struct EmuParams {
   EvenOdd<NP> EO;
 };
 
-// out = M v for one line, M = D (TRANS false) or D^T (TRANS true), in double-float
-template <int NP, bool TRANS>
+// Whether an order runs its line products and factor scaling in packed form (DOT: with the fused
+// reduction of a CG step, whose registers come on top).  Measured, GDOF/s at 1.6e7 nodes, scalar /
+// packed: plain N = 2 59 / 57, 4 52 / 51, 10 32 / 30, 7 42 / 44.5, 11 20.6 / 24.6, 15 17 / 26; DOT
+// N = 5 43 / 37, 6 36 / 36, 7 42 / 40, 8 35.5 / 28, 9 27 / 30, 15 14.5 / 21.
+__host__ __device__ constexpr bool emu_packed(int NP, bool dot) {
+  return NP == 4 || NP == 10 || NP >= 12 || (!dot && NP >= 6 && NP <= 9);
+}
+// whether the even and odd parts of a line are formed together too (N = 15 without 26, with 22 GDOF/s)
+__host__ __device__ constexpr bool emu_packed_parts(int NP) { return NP <= 14; }
+
+// out = M v for one line, M = D (TRANS false) or D^T (TRANS true), in double-float: the odd part
+// (p_i, from o) and the even part (q_i, from e), accumulated together in the two halves of packed
+// operations or one after the other.  Odd n adds the middle node mid = N / 2: M[i][mid] v_mid joins
+// q_i (mirrored with a sign like q), and the middle row, M[mid][mid] = 0 and
+// M[mid][N-m] = -M[mid][m], is sum_m M[mid][m] o_m.
+template <int NP, bool TRANS, bool PK>
 __device__ __forceinline__ void df_line(const EmuParams<NP> &P, const float2 (&v)[NP], float2 (&out)[NP]) {
-  if constexpr (NP % 2 == 0) {
-    constexpr int H = NP / 2;
-    const float *aph = TRANS ? P.EO.bph : P.EO.aph, *apl = TRANS ? P.EO.bpl : P.EO.apl;
-    const float *amh = TRANS ? P.EO.bmh : P.EO.amh, *aml = TRANS ? P.EO.bml : P.EO.aml;
-    float2 ev[H], od[H];
+  constexpr int H = NP / 2, MID = NP / 2, T = TRANS ? 1 : 0;
+  const float2 *ah = P.EO.hi[T], *al = P.EO.lo[T];
+  float2 oeh[H], oel[H];  // (o, e): high words, low words
 #pragma unroll
-    for (int m = 0; m < H; ++m) {
-      ev[m] = dpm(v[m], v[NP - 1 - m], false);
-      od[m] = dpm(v[m], v[NP - 1 - m], true);
+  for (int m = 0; m < H; ++m) {
+    const float2 va = v[m], vb = v[NP - 1 - m];
+    if constexpr (PK && emu_packed_parts(NP)) {  // va - vb and va + vb at once, as dpm
+      const float2 a2 = make_float2(va.x, va.x), b2 = make_float2(-vb.x, vb.x);
+      const float2 t = __fadd2_rn(a2, b2), z = sub2(t, a2);
+      const float2 err = __fadd2_rn(sub2(a2, sub2(t, z)), sub2(b2, z));
+      oeh[m] = t;
+      oel[m] = __fadd2_rn(__fadd2_rn(make_float2(va.y, va.y), make_float2(-vb.y, vb.y)), err);
+    } else {
+      const float2 e = dpm(va, vb, false), o = dpm(va, vb, true);
+      oeh[m] = make_float2(o.x, e.x);
+      oel[m] = make_float2(o.y, e.y);
     }
+  }
 #pragma unroll
-    for (int i = 0; i < H; ++i) {
-      float sp, cp, sq, cq;
-      dacc_first(sp, cp, aph[i * H], apl[i * H], od[0]);
-      dacc_first(sq, cq, amh[i * H], aml[i * H], ev[0]);
+  for (int i = 0; i < H; ++i) {
+    float2 s, c;
+    if constexpr (PK) {
+      dacc2_first(s, c, ah[i * H], al[i * H], oeh[0], oel[0]);
+#pragma unroll
+      for (int m = 1; m < H; ++m) dacc2(s, c, ah[i * H + m], al[i * H + m], oeh[m], oel[m]);
+    } else {
+      dacc_first(s.x, c.x, ah[i * H].x, al[i * H].x, make_float2(oeh[0].x, oel[0].x));
+      dacc_first(s.y, c.y, ah[i * H].y, al[i * H].y, make_float2(oeh[0].y, oel[0].y));
 #pragma unroll
       for (int m = 1; m < H; ++m) {
-        dacc(sp, cp, aph[i * H + m], apl[i * H + m], od[m]);
-        dacc(sq, cq, amh[i * H + m], aml[i * H + m], ev[m]);
+        dacc(s.x, c.x, ah[i * H + m].x, al[i * H + m].x, make_float2(oeh[m].x, oel[m].x));
+        dacc(s.y, c.y, ah[i * H + m].y, al[i * H + m].y, make_float2(oeh[m].y, oel[m].y));
       }
-      out[i] = dcombine(sp, cp, sq, cq, false);
-      out[NP - 1 - i] = dcombine(sp, cp, sq, cq, true);
     }
-  } else if constexpr (NP >= 3) {
-    // odd n: the same pairs around the middle node mid = N / 2, plus its own terms: M[i][mid] v_mid
-    // joins q_i (mirrored with a sign like q), and the middle row, M[mid][mid] = 0 and
-    // M[mid][N-m] = -M[mid][m], is sum_m M[mid][m] o_m
-    constexpr int H = NP / 2, MID = NP / 2;
-    const float *aph = TRANS ? P.EO.bph : P.EO.aph, *apl = TRANS ? P.EO.bpl : P.EO.apl;
-    const float *amh = TRANS ? P.EO.bmh : P.EO.amh, *aml = TRANS ? P.EO.bml : P.EO.aml;
-    const float *Dh = P.D.hi, *Dl = P.D.lo;
-    float2 ev[H], od[H];
-#pragma unroll
-    for (int m = 0; m < H; ++m) {
-      ev[m] = dpm(v[m], v[NP - 1 - m], false);
-      od[m] = dpm(v[m], v[NP - 1 - m], true);
-    }
-#pragma unroll
-    for (int i = 0; i < H; ++i) {
-      float sp, cp, sq, cq;
-      dacc_first(sp, cp, aph[i * H], apl[i * H], od[0]);
-      dacc_first(sq, cq, amh[i * H], aml[i * H], ev[0]);
-#pragma unroll
-      for (int m = 1; m < H; ++m) {
-        dacc(sp, cp, aph[i * H + m], apl[i * H + m], od[m]);
-        dacc(sq, cq, amh[i * H + m], aml[i * H + m], ev[m]);
-      }
+    if constexpr (NP % 2 == 1) {
       const int qm = TRANS ? MID * NP + i : i * NP + MID;  // M[i][mid]
-      dacc(sq, cq, Dh[qm], Dl[qm], v[MID]);
-      out[i] = dcombine(sp, cp, sq, cq, false);
-      out[NP - 1 - i] = dcombine(sp, cp, sq, cq, true);
+      dacc(s.y, c.y, P.D.hi[qm], P.D.lo[qm], v[MID]);
     }
+    out[i] = dcombine(s.x, c.x, s.y, c.y, false);
+    out[NP - 1 - i] = dcombine(s.x, c.x, s.y, c.y, true);
+  }
+  if constexpr (NP % 2 == 1) {
     float s, c;
-    dacc_first(s, c, Dh[TRANS ? MID : MID * NP], Dl[TRANS ? MID : MID * NP], od[0]);
+    dacc_first(s, c, P.D.hi[TRANS ? MID : MID * NP], P.D.lo[TRANS ? MID : MID * NP], make_float2(oeh[0].x, oel[0].x));
 #pragma unroll
     for (int m = 1; m < H; ++m) {
       const int q = TRANS ? m * NP + MID : MID * NP + m;  // M[mid][m]
-      dacc(s, c, Dh[q], Dl[q], od[m]);
+      dacc(s, c, P.D.hi[q], P.D.lo[q], make_float2(oeh[m].x, oel[m].x));
     }
     out[MID] = dnorm(s, c);
   }
 }
 
-__host__ __device__ constexpr int emu_eb(int NP) {
+// elements per block: with the factor block staged, and with factors read directly (there the block's
+// last warp is filled up as far as shared memory lets two blocks or more onto an SM: N = 5 with 7
+// elements 48 GDOF/s against 46 with 5, 6 with 5 43 / 36 with 3, 8 with 3 36.5 / 33.5 with 1, 9 with
+// 3 31.6 / 29.6 with 1)
+__host__ __device__ constexpr int emu_eb_staged(int NP) {
   return NP <= 2 ? 32 : NP == 3 ? 14 : NP == 4 ? 8 : NP == 5 ? 5 : NP == 6 ? 3 : NP <= 8 ? 2 : 1;
 }
-
-template <int NP>
-struct EmuCfg {
-  static constexpr int NP2 = NP * NP, NP3 = NP2 * NP, EB = emu_eb(NP), NT = NP2 * EB;
-  static constexpr int RS = NP | 1, PS = NP * RS, BUF = NP * PS;
-  static constexpr int GS = (12 * NP3 + 3) / 4 * 4;  // factor block of one element (floats)
-  // the factor block can be staged in shared memory by one bulk (TMA) copy when it fits
-  static constexpr bool STAGE_FITS = (size_t)EB * (GS * sizeof(float) + 3 * BUF * sizeof(float2)) <= 112 * 1024;
-  // byte offsets: [factor block (TMA, offset 0)] [value buffers] [reduction slots, mbarrier]
-  static constexpr size_t buf_off(bool stage) { return stage ? (size_t)EB * GS * sizeof(float) : 0; }
-  static constexpr size_t red_off(bool stage) {
-    return (buf_off(stage) + (size_t)EB * 3 * BUF * sizeof(float2) + 15) / 16 * 16;
-  }
-  // reduction slots (32 doubles), mbarrier, flag, per-element exponent maxima (EB ints)
-  static constexpr size_t smem(bool stage) { return red_off(stage) + 32 * 8 + 16 + 16 + (size_t)EB * 4; }
-};
-
-// blocks per SM the register allocation is held to at high order (one element per block would
-// otherwise leave one or two blocks on an SM); 0 = no floor (an explicit 1 lets the compiler take
-// far more registers, and at N = 7 a floor of 5 or 6 blocks measured slower than none)
-__host__ __device__ constexpr int emu_min_blocks(int NP) {
-  return NP == 10 ? 4 : NP == 11 ? 3 : NP >= 12 ? 2 : 0;
+__host__ __device__ constexpr int emu_eb(int NP) {
+  return NP == 6 ? 7 : NP == 7 ? 5 : (NP == 9 || NP == 10) ? 3 : NP == 12 ? 2 : emu_eb_staged(NP);
 }
 
-// DOT: the fused (u, y) reduction of the CG step (pAp) is compiled in and runs when P.partials is
-// set.  Plain applies use DOT = false (no reduction code; 5-10% faster from N = 8 on) except at
-// N = 7, where the kernel that carries the code measured 6% faster (it is scheduled differently).
-__host__ __device__ constexpr bool emu_plain_has_dot(int NP) { return NP == 8; }
+template <int NP, bool STAGE>
+struct EmuCfg {
+  static constexpr int NP2 = NP * NP, NP3 = NP2 * NP, EB = STAGE ? emu_eb_staged(NP) : emu_eb(NP), NT = NP2 * EB;
+  static constexpr int RS = NP | 1, PS = NP * RS, BUF = NP * PS;
+  static constexpr int GS = (12 * NP3 + 3) / 4 * 4;  // factor block of one element (floats)
+  // byte offsets: [factor block (TMA, offset 0)] [value buffers] [reduction slots, mbarrier]
+  static constexpr size_t BUF_OFF = STAGE ? (size_t)EB * GS * sizeof(float) : 0;
+  static constexpr size_t RED_OFF = (BUF_OFF + (size_t)EB * 3 * BUF * sizeof(float2) + 15) / 16 * 16;
+  // reduction slots (32 doubles), mbarrier, flag, per-element exponent maxima (EB ints)
+  static constexpr size_t SMEM = RED_OFF + 32 * 8 + 16 + 16 + (size_t)EB * 4;
+};
+// the factor block can be staged in shared memory by one bulk (TMA) copy when it fits
+__host__ __device__ constexpr bool emu_stage_fits(int NP) {
+  return (size_t)emu_eb_staged(NP) * ((12 * NP * NP * NP + 3) / 4 * 4 * sizeof(float) +
+                                      3 * NP * NP * (NP | 1) * sizeof(float2)) <= 112 * 1024;
+}
+
+// Blocks per SM the register allocation is held to; 0 = no floor (an explicit 1 lets the compiler
+// take far more registers).  Measured for the packed forms over floors of 0..7.
+__host__ __device__ constexpr int emu_min_blocks(int NP, bool stage, bool dot) {
+  if (stage) return NP == 10 ? 4 : NP == 11 ? 3 : NP >= 12 ? 2 : 0;
+  if (dot) return NP == 4 ? 7 : NP == 10 || NP >= 12 ? 2 : 0;
+  return NP == 4 ? 7 : NP == 6 || NP == 7 ? 4 : NP == 8 ? 5 : NP == 9 || NP == 11 ? 3 : NP >= 10 ? 2 : 0;
+}
 
 // How the line products of phases 1 and 3 are laid out in code: 0 three inlined line products per
 // phase; 2 the r- and s-lines through one loop body, the t-line (the thread's column, in
 // registers) inlined; 3 all three directions through one loop body (the t-line read from shared
 // memory).  The loops shorten the code (fewer instruction-fetch stalls) at some addressing cost.
-// Measured on GB300 (GDOF/s; 64^3 mesh, 48^3 at N = 12..14; forms 0 / 2 / 3): N = 3 56 / 57.2 /
-// 52, 5 41.1 / 42.5 / 41, 7 38.5 / 43.7 / 40.4, 8 28.5 / 33.2 / 30.0, 9 28.7 / 28.5 / 22,
-// 10 31.0 / 33.6 / 26.0, 11 15.6 / 21.0 / 18.4, 12 16.7 / 20.6 / 20.4, 13 17.0 / 11.3 / 17.1,
-// 14 15.1 / 10.3 / 16.9, 15 11.6 / 9.2 / 18.0.
+// Packed forms, GDOF/s at 1.6e7 nodes, modes 0 / 2 / 3: N = 3 61 / 59 / 55, 5 48 / 47 / 45, 6 41 / 43 /
+// 40, 7 41.5 / 44.5 / 40, 8 34.5 / 36.5 / 35, 9 31.6 / 31.0 / 30.8, 11 23.5 / 24.6 / 23.7, 12 23.5 / 19 /
+// 19, 13 16 / 17 / 20, 14 19 / 12 / 24, 15 16 / 13 / 26.
 __host__ __device__ constexpr int emu_loop_mode(int NP) {
-  return (NP == 4 || NP == 6 || NP == 8 || NP == 9 || NP == 11 || NP == 12 || NP == 13) ? 2 : NP >= 14 ? 3 : 0;
+  return NP >= 14 ? 3 : (NP == 7 || NP == 8 || NP == 9 || NP == 11 || NP == 12) ? 2 : 0;
 }
 
+// the block's factors asked for in L2 at its start by one bulk prefetch (one element per block and
+// two blocks per SM leave the loads exposed: N = 13 16.9 -> 19.9, 15 24.3 -> 26.2 GDOF/s; slower
+// below)
+__host__ __device__ constexpr bool emu_prefetch(int NP) { return NP >= 14; }
+
 template <int NP, bool BOXM, bool STAGE, bool DOT>
-__global__ void __launch_bounds__(EmuCfg<NP>::NT, emu_min_blocks(NP)) k_apply_emu(const EmuParams<NP> P) {
-  using C = EmuCfg<NP>;
+__global__ void __launch_bounds__(EmuCfg<NP, STAGE>::NT, emu_min_blocks(NP, STAGE, DOT)) k_apply_emu(const EmuParams<NP> P) {
+  using C = EmuCfg<NP, STAGE>;
   constexpr int N = NP - 1, NP2 = C::NP2, NP3 = C::NP3, EB = C::EB, NT = C::NT, RS = C::RS, PS = C::PS,
                 BUF = C::BUF, GS = C::GS;
+  constexpr bool PK = emu_packed(NP, DOT);
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  static_assert(C::buf_off(STAGE) % 16 == 0 && C::red_off(STAGE) % 16 == 0, "shared-memory alignment");
+  static_assert(C::BUF_OFF % 16 == 0 && C::RED_OFF % 16 == 0, "shared-memory alignment");
   float *sG = reinterpret_cast<float *>(smem_raw);  // TMA destination: 16-byte aligned at offset 0
-  float2 *sbuf = reinterpret_cast<float2 *>(smem_raw + C::buf_off(STAGE));
-  double *s_red = reinterpret_cast<double *>(smem_raw + C::red_off(STAGE));
+  float2 *sbuf = reinterpret_cast<float2 *>(smem_raw + C::BUF_OFF);
+  double *s_red = reinterpret_cast<double *>(smem_raw + C::RED_OFF);
   uint64_t *bar = reinterpret_cast<uint64_t *>(s_red + 32);
   int *s_flag = reinterpret_cast<int *>(bar + 1);
   int *s_emax = s_flag + 4;  // [EB] largest biased FP64 exponent of each element's u
@@ -347,6 +387,15 @@ __global__ void __launch_bounds__(EmuCfg<NP>::NT, emu_min_blocks(NP)) k_apply_em
     if (tid == 0) {
       const int64_t nel = (P.E - e0) < EB ? (P.E - e0) : EB;
       tma_load_1d(sG, P.Gf + e0 * P.gs, (uint32_t)(nel * P.gs * sizeof(float)), bar);
+    }
+  }
+
+  if constexpr (!STAGE && emu_prefetch(NP)) {
+    if (tid == 0) {
+      const int64_t nel = (P.E - e0) < EB ? (P.E - e0) : EB;
+      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(P.Gf + e0 * P.gs),
+                   "r"((uint32_t)(nel * P.gs * sizeof(float)))
+                   : "memory");
     }
   }
 
@@ -424,7 +473,7 @@ __global__ void __launch_bounds__(EmuCfg<NP>::NT, emu_min_blocks(NP)) k_apply_em
       float2 row[NP], out[NP];
 #pragma unroll
       for (int m = 0; m < NP; ++m) row[m] = su[ib + m * is];
-      df_line<NP, false>(P, row, out);
+      df_line<NP, false, PK>(P, row, out);
       if (dir == 2) {
 #pragma unroll
         for (int k = 0; k < NP; ++k) wt[k] = out[k];
@@ -438,7 +487,7 @@ __global__ void __launch_bounds__(EmuCfg<NP>::NT, emu_min_blocks(NP)) k_apply_em
     // the t-line (the column, in registers) inlined; the r-line (j = a, k = b) into sr and the
     // s-line (i = a, k = b) into ss through one loop body (the same base and stride address input
     // and output)
-    df_line<NP, false>(P, uc, wt);  // u_t of the column
+    df_line<NP, false, PK>(P, uc, wt);  // u_t of the column
 #pragma unroll 1
     for (int dir = 0; dir < 2; ++dir) {
       const int ib = dir == 0 ? b * PS + a * RS : b * PS + a;
@@ -447,21 +496,21 @@ __global__ void __launch_bounds__(EmuCfg<NP>::NT, emu_min_blocks(NP)) k_apply_em
       float2 row[NP], out[NP];
 #pragma unroll
       for (int m = 0; m < NP; ++m) row[m] = su[ib + m * is];
-      df_line<NP, false>(P, row, out);
+      df_line<NP, false, PK>(P, row, out);
 #pragma unroll
       for (int i = 0; i < NP; ++i) dst[ib + i * is] = out[i];
     }
   } else {
-    df_line<NP, false>(P, uc, wt);  // u_t of the column
+    df_line<NP, false, PK>(P, uc, wt);  // u_t of the column
     float2 row[NP], out[NP];
 #pragma unroll
     for (int m = 0; m < NP; ++m) row[m] = su[b * PS + a * RS + m];
-    df_line<NP, false>(P, row, out);
+    df_line<NP, false, PK>(P, row, out);
 #pragma unroll
     for (int i = 0; i < NP; ++i) sr[b * PS + a * RS + i] = out[i];
 #pragma unroll
     for (int m = 0; m < NP; ++m) row[m] = su[b * PS + m * RS + a];
-    df_line<NP, false>(P, row, out);
+    df_line<NP, false, PK>(P, row, out);
 #pragma unroll
     for (int j = 0; j < NP; ++j) ss[b * PS + j * RS + a] = out[j];
   }
@@ -478,16 +527,49 @@ __global__ void __launch_bounds__(EmuCfg<NP>::NT, emu_min_blocks(NP)) k_apply_em
     return;
   }
   const float *Ge = STAGE ? (sG + es * GS + t2) : (P.Gf + (active ? e : 0) * P.gs + t2);
-#pragma unroll
-  for (int k = 0; k < NP; ++k) {
-    const int q = k * PS + b * RS + a;
-    const int o = k * NP2;
-    float gh[6], gl[6];
+  auto load_g = [&](int k, float(&gh)[6], float(&gl)[6]) {
 #pragma unroll
     for (int f = 0; f < 6; ++f) {
-      gh[f] = (STAGE || active) ? Ge[(2 * f) * NP3 + o] : 0.f;
-      gl[f] = (STAGE || active) ? Ge[(2 * f + 1) * NP3 + o] : 0.f;
+      gh[f] = (STAGE || active) ? Ge[(2 * f) * NP3 + k * NP2] : 0.f;
+      gl[f] = (STAGE || active) ? Ge[(2 * f + 1) * NP3 + k * NP2] : 0.f;
     }
+  };
+  // two nodes of the column at a time, one in each half of the packed operations
+  constexpr int KP = PK ? NP / 2 * 2 : 0;
+#pragma unroll
+  for (int k = 0; k < KP; k += 2) {
+    const int q0 = k * PS + b * RS + a, q1 = q0 + PS;
+    float g0h[6], g0l[6], g1h[6], g1l[6];
+    load_g(k, g0h, g0l);
+    load_g(k + 1, g1h, g1l);
+    const float2 r0 = sr[q0], r1 = sr[q1], s0 = ss[q0], s1 = ss[q1], t0 = wt[k], t1 = wt[k + 1];
+    const float2 vh[3] = {make_float2(r0.x, r1.x), make_float2(s0.x, s1.x), make_float2(t0.x, t1.x)};
+    const float2 vl[3] = {make_float2(r0.y, r1.y), make_float2(s0.y, s1.y), make_float2(t0.y, t1.y)};
+    constexpr int F[3][3] = {{0, 1, 2}, {1, 3, 4}, {2, 4, 5}};
+    float2 w0[3], w1[3];
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      float2 s, c;
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        const float2 gh = make_float2(g0h[F[r][d]], g1h[F[r][d]]), gl = make_float2(g0l[F[r][d]], g1l[F[r][d]]);
+        if (d == 0)
+          dacc2_first(s, c, gh, gl, vh[d], vl[d]);
+        else
+          dacc2(s, c, gh, gl, vh[d], vl[d]);
+      }
+      w0[r] = dnorm(s.x, c.x);
+      w1[r] = dnorm(s.y, c.y);
+    }
+    sr[q0] = w0[0], sr[q1] = w1[0];
+    ss[q0] = w0[1], ss[q1] = w1[1];
+    wt[k] = w0[2], wt[k + 1] = w1[2];
+  }
+#pragma unroll
+  for (int k = KP; k < NP; ++k) {  // one node at a time: the last of an odd column, or all
+    const int q = k * PS + b * RS + a;
+    float gh[6], gl[6];
+    load_g(k, gh, gl);
     const float2 ur = sr[q], us = ss[q], ut = wt[k];
     float s, c;
     dacc_first(s, c, gh[0], gl[0], ur);
@@ -516,7 +598,7 @@ __global__ void __launch_bounds__(EmuCfg<NP>::NT, emu_min_blocks(NP)) k_apply_em
       float2 row[NP], out[NP];
 #pragma unroll
       for (int m = 0; m < NP; ++m) row[m] = dir == 2 ? wt[m] : buf[ib + m * is];
-      df_line<NP, true>(P, row, out);
+      df_line<NP, true, PK>(P, row, out);
       if (dir == 2) {
 #pragma unroll
         for (int k = 0; k < NP; ++k) yt[k] = out[k];
@@ -526,7 +608,7 @@ __global__ void __launch_bounds__(EmuCfg<NP>::NT, emu_min_blocks(NP)) k_apply_em
       }
     }
   } else if constexpr (emu_loop_mode(NP) == 2) {
-    df_line<NP, true>(P, wt, yt);  // D^T w_t of the column
+    df_line<NP, true, PK>(P, wt, yt);  // D^T w_t of the column
     __syncthreads();
     // ---- phase 3: transposed contractions: 0 the r-line of sr, 1 the s-line of ss (in place) ----
 #pragma unroll 1
@@ -537,24 +619,24 @@ __global__ void __launch_bounds__(EmuCfg<NP>::NT, emu_min_blocks(NP)) k_apply_em
       float2 row[NP], out[NP];
 #pragma unroll
       for (int m = 0; m < NP; ++m) row[m] = buf[ib + m * is];
-      df_line<NP, true>(P, row, out);
+      df_line<NP, true, PK>(P, row, out);
 #pragma unroll
       for (int i = 0; i < NP; ++i) buf[ib + i * is] = out[i];
     }
   } else {
-    df_line<NP, true>(P, wt, yt);  // D^T w_t of the column
+    df_line<NP, true, PK>(P, wt, yt);  // D^T w_t of the column
     __syncthreads();
 
     // ---- phase 3: transposed r and s contractions ----
     float2 row[NP], out[NP];
 #pragma unroll
     for (int m = 0; m < NP; ++m) row[m] = sr[b * PS + a * RS + m];
-    df_line<NP, true>(P, row, out);
+    df_line<NP, true, PK>(P, row, out);
 #pragma unroll
     for (int i = 0; i < NP; ++i) sr[b * PS + a * RS + i] = out[i];
 #pragma unroll
     for (int m = 0; m < NP; ++m) row[m] = ss[b * PS + m * RS + a];
-    df_line<NP, true>(P, row, out);
+    df_line<NP, true, PK>(P, row, out);
 #pragma unroll
     for (int j = 0; j < NP; ++j) ss[b * PS + j * RS + a] = out[j];
   }
@@ -618,26 +700,27 @@ __global__ void __launch_bounds__(EmuCfg<NP>::NT, emu_min_blocks(NP)) k_apply_em
 }
 
 template <int NP, bool BOXM, bool STAGE, bool DOT>
-sem_status launch_k(const EmuParams<NP> &p, unsigned grid, cudaStream_t s) {
-  using C = EmuCfg<NP>;
+sem_status launch_k(const EmuParams<NP> &p, cudaStream_t s) {
+  using C = EmuCfg<NP, STAGE>;
+  const unsigned grid = (unsigned)((p.E + C::EB - 1) / C::EB);
+  if (p.partials && grid > SEM_MAX_PARTIALS) return sem_fail(SEM_ERR_INVALID, "too many elements for fused dot");
   static std::atomic<unsigned long long> attr_done;
-  const cudaError_t e = set_smem_limit_once(k_apply_emu<NP, BOXM, STAGE, DOT>, C::smem(STAGE), attr_done);
+  const cudaError_t e = set_smem_limit_once(k_apply_emu<NP, BOXM, STAGE, DOT>, C::SMEM, attr_done);
   if (e != cudaSuccess) return sem_fail(SEM_ERR_CUDA, std::string("emu attributes: ") + cudaGetErrorString(e));
-  k_apply_emu<NP, BOXM, STAGE, DOT><<<grid, C::NT, C::smem(STAGE), s>>>(p);
+  k_apply_emu<NP, BOXM, STAGE, DOT><<<grid, C::NT, C::SMEM, s>>>(p);
   return SEM_OK;
 }
 
 template <int NP, bool STAGE>
-sem_status launch_b(const EmuParams<NP> &p, bool boxm, bool dot, unsigned grid, cudaStream_t s) {
-  if (dot || emu_plain_has_dot(NP))
-    return boxm ? launch_k<NP, true, STAGE, true>(p, grid, s) : launch_k<NP, false, STAGE, true>(p, grid, s);
-  return boxm ? launch_k<NP, true, STAGE, false>(p, grid, s) : launch_k<NP, false, STAGE, false>(p, grid, s);
+sem_status launch_b(const EmuParams<NP> &p, bool boxm, bool dot, cudaStream_t s) {
+  if (dot)
+    return boxm ? launch_k<NP, true, STAGE, true>(p, s) : launch_k<NP, false, STAGE, true>(p, s);
+  return boxm ? launch_k<NP, true, STAGE, false>(p, s) : launch_k<NP, false, STAGE, false>(p, s);
 }
 
 template <int NP>
 sem_status launch_emu(const sem_handle *h, const double *u, double *y, double *partials, SemScalars *scal,
                       cudaStream_t s) {
-  using C = EmuCfg<NP>;
   EmuParams<NP> p;
   p.E = h->E;
   p.sx = h->box[0];
@@ -669,26 +752,22 @@ sem_status launch_emu(const sem_handle *h, const double *u, double *y, double *p
     hi = (float)x;
     lo = (float)(x - (double)hi);
   };
-  for (int i = 0; i < H && NP >= 2; ++i)  // pairs (i, N - i), i < H = n / 2, for even and odd n
-    for (int m = 0; m < H; ++m) {
-      const double *D = h->D64h;
-      const int N = NP - 1;
-      split(0.5 * (D[i * NP + m] + D[(N - i) * NP + m]), p.EO.aph[i * H + m], p.EO.apl[i * H + m]);
-      split(0.5 * (D[i * NP + m] - D[(N - i) * NP + m]), p.EO.amh[i * H + m], p.EO.aml[i * H + m]);
-      split(0.5 * (D[m * NP + i] + D[m * NP + (N - i)]), p.EO.bph[i * H + m], p.EO.bpl[i * H + m]);
-      split(0.5 * (D[m * NP + i] - D[m * NP + (N - i)]), p.EO.bmh[i * H + m], p.EO.bml[i * H + m]);
-    }
-  const unsigned grid = (unsigned)((p.E + C::EB - 1) / C::EB);
-  if (partials && grid > SEM_MAX_PARTIALS) return sem_fail(SEM_ERR_INVALID, "too many elements for fused dot");
+  for (int t = 0; t < 2; ++t)  // M = D, D^T; pairs (i, N - i), i < H = n / 2, for even and odd n
+    for (int i = 0; i < H && NP >= 2; ++i)
+      for (int m = 0; m < H; ++m) {
+        const double *D = h->D64h;
+        const int N = NP - 1, q = i * H + m;
+        const double u = t == 0 ? D[i * NP + m] : D[m * NP + i], v = t == 0 ? D[(N - i) * NP + m] : D[m * NP + (N - i)];
+        split(0.5 * (u + v), p.EO.hi[t][q].x, p.EO.lo[t][q].x);
+        split(0.5 * (u - v), p.EO.hi[t][q].y, p.EO.lo[t][q].y);
+      }
   if (partials && !scal) return sem_fail(SEM_ERR_INVALID, "fused dot needs the solver scalars");
   const bool boxm = p.glo == nullptr && p.bc != SEM_BC_MASK;
-  // variant 0: factor block staged by TMA when it fits; other variants read factors directly;
-  // automatic (-1): direct reads, except at N = 5 where staging measured faster on GB300
-  const int variant = h->apply_variant < 0 ? (NP == 6 ? 0 : 1) : h->apply_variant;
-  const bool stage = C::STAGE_FITS && variant == 0;
-  sem_status st;
-  st = stage ? launch_b<NP, C::STAGE_FITS>(p, boxm, partials != nullptr, grid, s)
-             : launch_b<NP, false>(p, boxm, partials != nullptr, grid, s);
+  // variant 0: factor block staged by TMA when it fits; other variants, and automatic (-1), read
+  // factors directly
+  const bool stage = emu_stage_fits(NP) && h->apply_variant == 0;
+  const sem_status st = stage ? launch_b<NP, emu_stage_fits(NP)>(p, boxm, partials != nullptr, s)
+                              : launch_b<NP, false>(p, boxm, partials != nullptr, s);
   if (st != SEM_OK) return st;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return sem_fail(SEM_ERR_CUDA, std::string("emu apply launch: ") + cudaGetErrorString(e));
