@@ -257,9 +257,16 @@ __host__ __device__ constexpr size_t apply_red_off() {
          16 * 16;
 }
 
+// bytes of the reduction slots: 32 doubles (batched per-element sums) or one value per thread
+template <int NP, typename T, int EB>
+__host__ __device__ constexpr size_t apply_red_size() {
+  constexpr size_t per_thread = ((size_t)ApplyCfg<NP, EB>::NT * sizeof(T) + 15) / 16 * 16;
+  return per_thread > 32 * 8 ? per_thread : 32 * 8;
+}
+
 template <int NP, typename T, int EB, bool STAGE, typename TG = T>
 __host__ __device__ constexpr size_t apply_smem() {
-  return apply_red_off<NP, T, EB, STAGE, TG>() + 32 * 8 + 16 + 16;
+  return apply_red_off<NP, T, EB, STAGE, TG>() + apply_red_size<NP, T, EB>() + 16;
 }
 
 // BOXM: structured box numbering with no mask array (bc NONE or BOX): global ids and Dirichlet
@@ -294,8 +301,7 @@ __global__ void __launch_bounds__(ApplyCfg<NP, EB_>::NT, apply_min_blocks<T>(NP,
   TG *sG = reinterpret_cast<TG *>(smem_raw);  // TMA destination: 16-byte aligned at offset 0
   T *sbuf = reinterpret_cast<T *>(smem_raw + (STAGE ? EB * GS * sizeof(TG) : 0));
   double *s_red = reinterpret_cast<double *>(smem_raw + RED_OFF);
-  uint64_t *bar = reinterpret_cast<uint64_t *>(s_red + 32);
-  int *s_flag = reinterpret_cast<int *>(bar + 1);
+  uint64_t *bar = reinterpret_cast<uint64_t *>(smem_raw + RED_OFF + apply_red_size<NP, T, EB_>());
 
   // inside a solve: nothing to do once the iteration has stopped (flag set by an earlier launch)
   if (P.scal && (P.scal->converged || P.scal->breakdown)) return;
@@ -466,7 +472,7 @@ __global__ void __launch_bounds__(ApplyCfg<NP, EB_>::NT, apply_min_blocks<T>(NP,
     const OtfColumn oc =
         otf_column(reinterpret_cast<const float *>(c_Gf) + eo * SEM_OTF_STRIDE, P.gll.x[a], P.gll.x[b]);
     const float wab = P.gll.w[a] * P.gll.w[b];
-    const float *kp = c_kap ? c_kap + eo * NP3 + t2 : nullptr;
+    const int64_t ko = eo * NP3 + t2;
 #pragma unroll
     for (int k = 0; k < NP; ++k) {
       const int q = k * PS + b * RS + a;
@@ -480,7 +486,7 @@ __global__ void __launch_bounds__(ApplyCfg<NP, EB_>::NT, apply_min_blocks<T>(NP,
       }
       const float det = oc.d0 + t * (oc.d1 + t * oc.d2);
       float num = wab * P.gll.w[k];
-      if (kp) num *= kp[k * NP2];
+      if (c_kap) num *= c_kap[ko + k * NP2];
       const float sc = __fdividef(num, det);
       const float ur = sr[q], us = ss[q], ut = wt[k];
       float qv[3];
@@ -553,38 +559,60 @@ __global__ void __launch_bounds__(ApplyCfg<NP, EB_>::NT, apply_min_blocks<T>(NP,
   __syncthreads();
 
   // ---- phase 4: assemble the column and scatter y += M Q^T y_e ----
-  T dotp = T(0);
-  if constexpr (BOXM) {
-    const int64_t plane = c_gxs * c_gys;
-    T *yp = c_y + gbase;
-    const bool ij_interior = (a > 0) && (a < N) && (b > 0) && (b < N);
-#pragma unroll
-    for (int k = 0; k < NP; ++k) {
-      const int q = k * PS + b * RS + a;
-      T yk = yc[k] + sr[q] + ss[q];
-      if (c_wJa && active) yk += c_wJa[el * NP3 + t2 + NP2 * k] * uc[k];
-      if ((dirbits >> k) & 1u) continue;
-      if (P.partials || P.pAp_batch) dotp += uc[k] * yk;
+  const bool ij_interior = (a > 0) && (a < N) && (b > 0) && (b < N) && (BOXM || !P.glo);
+  auto scatter = [&](int k, T yk) {
+    if constexpr (BOXM) {
+      T *yp = c_y + gbase;
+      const int64_t plane = c_gxs * c_gys;
       if (k > 0 && k < N && ij_interior)
         yp[k * plane] = yk;  // element-interior node: owned by this element alone
       else
         atomicAdd(yp + k * plane, yk);
-    }
-  } else if (active) {
-    const bool ij_interior = (a > 0) && (a < N) && (b > 0) && (b < N) && !P.glo;
-#pragma unroll
-    for (int k = 0; k < NP; ++k) {
-      if ((dirbits >> k) & 1u) continue;
-      const int q = k * PS + b * RS + a;
-      T yk = yc[k] + sr[q] + ss[q];
-      if (P.wJa) yk += P.wJa[e * NP3 + t2 + NP2 * k] * uc[k];
+    } else {
       const int64_t g = P.glo ? (int64_t)P.glo[e * NP3 + t2 + NP2 * k] : gbase + P.gxs * P.gys * k;
-      if (P.partials) dotp += uc[k] * yk;
       if (ij_interior && k > 0 && k < N)
         P.y[g] = yk;
       else
         atomicAdd(P.y + g, yk);
     }
+  };
+  // Optional arrays are tested through their own pointers, here and for kappa above: a pointer that was
+  // offset first ("q ? q + i : nullptr") and then tested was dereferenced with q null in the FP64 form
+  // of this kernel, where a build of the same source for the host is clean.
+  if (P.partials) {
+    // p^T A p and the CG step length: one warp adds the block's terms and publishes them before its
+    // scatter, so that its fences have no writes to wait for and the other warps do not wait at all
+    T dotp = T(0);
+#pragma unroll
+    for (int k = 0; k < NP; ++k) {
+      const int q = k * PS + b * RS + a;
+      yc[k] += sr[q] + ss[q];
+      if (c_wJa && active) yc[k] += c_wJa[el * NP3 + t2 + NP2 * k] * uc[k];
+      if (!((dirbits >> k) & 1u)) dotp += uc[k] * yc[k];
+    }
+    T *s_dot = reinterpret_cast<T *>(s_red);
+    s_dot[tid] = dotp;
+    __syncthreads();
+    if (tid < 32) {
+      double pAp;
+      if (warp_publish_2level(warp_sum(s_dot, NT), P.partials, P.gpartials, P.gtickets, &P.scal->counter[0], &pAp) &&
+          tid == 0)
+        cg_set_alpha(P.scal, pAp);
+    }
+#pragma unroll
+    for (int k = 0; k < NP; ++k)
+      if (!((dirbits >> k) & 1u)) scatter(k, yc[k]);
+    return;
+  }
+  T dotp = T(0);
+#pragma unroll
+  for (int k = 0; k < NP; ++k) {
+    const int q = k * PS + b * RS + a;
+    T yk = yc[k] + sr[q] + ss[q];
+    if (c_wJa && active) yk += c_wJa[el * NP3 + t2 + NP2 * k] * uc[k];
+    if ((dirbits >> k) & 1u) continue;  // Dirichlet node, or no element in this slot
+    if (P.pAp_batch) dotp += uc[k] * yk;
+    scatter(k, yk);
   }
 
   // ---- batched: per-problem p^T A p, one atomic add per element ----
@@ -606,25 +634,6 @@ __global__ void __launch_bounds__(ApplyCfg<NP, EB_>::NT, apply_min_blocks<T>(NP,
     }
   }
 
-  // ---- optional fused p^T A p and CG step length ----
-  if (P.partials) {
-    const double bs = block_sum<NT>((double)dotp, s_red);
-    double pAp;
-    if (publish_partial_2level<NT>(bs, P.partials, P.gpartials, P.gtickets, &P.scal->counter[0], s_red, s_flag,
-                                   &pAp)) {
-      if (tid == 0) {
-        SemScalars *S = P.scal;
-        S->pAp = pAp;
-        if (!(pAp > 0.0) || !isfinite(pAp) || !isfinite(S->rz)) {
-          S->breakdown = 1;
-          S->alpha = 0.0;
-        } else {
-          S->alpha = S->rz / pAp;
-        }
-        S->counter[0] = 0;
-      }
-    }
-  }
 }
 
 // largest dynamic shared memory a block may use on sm_103 (227 KB)

@@ -42,7 +42,7 @@ __host__ __device__ constexpr int fused_buf(int NP) { return NP * NP * (NP | 1);
 __host__ __device__ constexpr size_t fused_red_off(int NP) {
   return ((size_t)fused_es(NP) * 3 * fused_buf(NP) * sizeof(float) + 15) / 16 * 16;
 }
-__host__ __device__ constexpr size_t fused_smem_np(int NP) { return fused_red_off(NP) + (size_t)fused_es(NP) * 8; }
+__host__ __device__ constexpr size_t fused_smem_np(int NP) { return fused_red_off(NP) + (size_t)FT * 4; }
 __host__ __device__ constexpr size_t fused_smem() {
   size_t m = 0;
   for (int s = 0; s < NSLOT; ++s) m = fused_smem_np(SLOT_NP[s]) > m ? fused_smem_np(SLOT_NP[s]) : m;
@@ -89,7 +89,7 @@ __device__ __forceinline__ void fused_apply_tile(const SlotParams &S, int64_t ti
   static_assert(EB >= 1 && ES * NP2 >= FT, "tile against the block");
   const DConst<NP, float> &D = tab_D<NP>();
   float *sbuf = reinterpret_cast<float *>(smem);
-  double *s_el = reinterpret_cast<double *>(smem + fused_red_off(NP));  // ES per-element sums
+  float *s_dot = reinterpret_cast<float *>(smem + fused_red_off(NP));  // one p^T A p term per thread
   const int tid = threadIdx.x;
   const int es = tid / NP2, t2 = tid - es * NP2, a = t2 % NP, b = t2 / NP;
   const int64_t e = tile * EB + es;
@@ -191,7 +191,6 @@ __device__ __forceinline__ void fused_apply_tile(const SlotParams &S, int64_t ti
 #pragma unroll
     for (int j = 0; j < NP; ++j) ss[b * PS + j * RS + a] = out[j];
   }
-  if (tid < ES) s_el[tid] = 0.0;
   __syncthreads();
 
   // ---- assemble the column, scatter y += Q^T y_e, p^T A p of the element ----
@@ -211,9 +210,27 @@ __device__ __forceinline__ void fused_apply_tile(const SlotParams &S, int64_t ti
     else
       atomicAdd(yp + k * plane, yk);
   }
-  atomicAdd(&s_el[es], (double)dotp);
+  s_dot[tid] = dotp;  // zero for threads past the tile's elements and for finished problems
   __syncthreads();
-  if (t2 == 0 && live) atomicAdd(&pAp[B.prob], s_el[es]);
+  // p^T A p of the tile's elements, added to their problems by as few FP64 additions as there are
+  // problems: a tile whose elements belong to one problem is one sum by one warp
+  const int first = S.tile_entry[tile];
+  if (first + 1 >= S.nbatch || S.batch[first + 1].elem_off >= (tile + 1) * EB) {
+    if (tid < 32) {
+      const double v = warp_sum(s_dot, EB * NP2);
+      if (tid == 0 && live) atomicAdd(&pAp[B.prob], v);
+    }
+  } else {
+    for (int el2 = tid >> 5; el2 < EB; el2 += FT / 32) {
+      const double v = warp_sum(s_dot + el2 * NP2, NP2);
+      const int64_t e2 = tile * EB + el2;
+      if ((tid & 31) == 0 && e2 < S.E) {
+        int q = first;
+        while (q + 1 < S.nbatch && S.batch[q + 1].elem_off <= e2) ++q;
+        if (!*S.batch[q].done) atomicAdd(&pAp[S.batch[q].prob], v);
+      }
+    }
+  }
 }
 
 struct FusedParams {
@@ -255,7 +272,7 @@ __device__ __forceinline__ bool grid_barrier(const FusedParams &P) {
           break;
         }
         if (*err) break;
-        __nanosleep(256);
+        __nanosleep(64);
       }
       if (!ok) atomicOr(P.err, 1);
     }
@@ -268,7 +285,7 @@ __device__ __forceinline__ bool grid_barrier(const FusedParams &P) {
 
 __global__ void __launch_bounds__(FT, 4) k_batch_step(const FusedParams P) {
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ double s_red[32];
+  __shared__ float s_part[2][FT];
   const int tid = threadIdx.x;
 
   // ---- A: batched apply over the tiles of every order group ----
@@ -331,11 +348,14 @@ __global__ void __launch_bounds__(FT, 4) k_batch_step(const FusedParams P) {
         rb += r * r;
       }
     }
-    const double A = block_sum<FT>((double)ra, s_red), Bs = block_sum<FT>((double)rb, s_red);
-    if (tid == 0) {
-      atomicAdd(P.rzn + p, A);
-      atomicAdd(P.rrn + p, Bs);
+    s_part[0][tid] = ra;
+    s_part[1][tid] = rb;
+    __syncthreads();
+    if (tid < 64) {
+      const double v = warp_sum(s_part[tid >> 5], FT);
+      if ((tid & 31) == 0) atomicAdd((tid == 0 ? P.rzn : P.rrn) + p, v);
     }
+    __syncthreads();  // the next chunk writes s_part
   }
   if (!grid_barrier(P)) return;
 

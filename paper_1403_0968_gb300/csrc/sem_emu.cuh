@@ -315,7 +315,7 @@ __host__ __device__ constexpr int emu_eb(int NP) {
   return NP == 6 ? 7 : NP == 7 ? 5 : (NP == 9 || NP == 10) ? 3 : NP == 12 ? 2 : emu_eb_staged(NP);
 }
 
-template <int NP, bool STAGE>
+template <int NP, bool STAGE, bool DOT>
 struct EmuCfg {
   static constexpr int NP2 = NP * NP, NP3 = NP2 * NP, EB = STAGE ? emu_eb_staged(NP) : emu_eb(NP), NT = NP2 * EB;
   static constexpr int RS = NP | 1, PS = NP * RS, BUF = NP * PS;
@@ -323,8 +323,10 @@ struct EmuCfg {
   // byte offsets: [factor block (TMA, offset 0)] [value buffers] [reduction slots, mbarrier]
   static constexpr size_t BUF_OFF = STAGE ? (size_t)EB * GS * sizeof(float) : 0;
   static constexpr size_t RED_OFF = (BUF_OFF + (size_t)EB * 3 * BUF * sizeof(float2) + 15) / 16 * 16;
-  // reduction slots (32 doubles), mbarrier, flag, per-element exponent maxima (EB ints)
-  static constexpr size_t SMEM = RED_OFF + 32 * 8 + 16 + 16 + (size_t)EB * 4;
+  // reduction slots (one double per thread with the fused reduction), mbarrier, per-element exponent
+  // maxima (EB ints)
+  static constexpr size_t RED_SIZE = DOT ? ((size_t)NT * 8 + 15) / 16 * 16 : 0;
+  static constexpr size_t SMEM = RED_OFF + RED_SIZE + 16 + (size_t)EB * 4;
 };
 // the factor block can be staged in shared memory by one bulk (TMA) copy when it fits
 __host__ __device__ constexpr bool emu_stage_fits(int NP) {
@@ -357,8 +359,8 @@ __host__ __device__ constexpr int emu_loop_mode(int NP) {
 __host__ __device__ constexpr bool emu_prefetch(int NP) { return NP >= 14; }
 
 template <int NP, bool BOXM, bool STAGE, bool DOT>
-__global__ void __launch_bounds__(EmuCfg<NP, STAGE>::NT, emu_min_blocks(NP, STAGE, DOT)) k_apply_emu(const EmuParams<NP> P) {
-  using C = EmuCfg<NP, STAGE>;
+__global__ void __launch_bounds__(EmuCfg<NP, STAGE, DOT>::NT, emu_min_blocks(NP, STAGE, DOT)) k_apply_emu(const EmuParams<NP> P) {
+  using C = EmuCfg<NP, STAGE, DOT>;
   constexpr int N = NP - 1, NP2 = C::NP2, NP3 = C::NP3, EB = C::EB, NT = C::NT, RS = C::RS, PS = C::PS,
                 BUF = C::BUF, GS = C::GS;
   constexpr bool PK = emu_packed(NP, DOT);
@@ -367,11 +369,10 @@ __global__ void __launch_bounds__(EmuCfg<NP, STAGE>::NT, emu_min_blocks(NP, STAG
   float *sG = reinterpret_cast<float *>(smem_raw);  // TMA destination: 16-byte aligned at offset 0
   float2 *sbuf = reinterpret_cast<float2 *>(smem_raw + C::BUF_OFF);
   double *s_red = reinterpret_cast<double *>(smem_raw + C::RED_OFF);
-  uint64_t *bar = reinterpret_cast<uint64_t *>(s_red + 32);
-  int *s_flag = reinterpret_cast<int *>(bar + 1);
-  int *s_emax = s_flag + 4;  // [EB] largest biased FP64 exponent of each element's u
+  uint64_t *bar = reinterpret_cast<uint64_t *>(smem_raw + C::RED_OFF + C::RED_SIZE);
+  int *s_emax = reinterpret_cast<int *>(bar + 2);  // [EB] largest biased FP64 exponent of each element's u
 
-  if (DOT && P.partials && (P.scal->converged || P.scal->breakdown)) return;
+  if (DOT && (P.scal->converged || P.scal->breakdown)) return;
   const int tid = threadIdx.x;
   const int es = tid / NP2, t2 = tid - es * NP2, a = t2 % NP, b = t2 / NP;
   if (t2 == 0) s_emax[es] = 1;
@@ -643,65 +644,78 @@ __global__ void __launch_bounds__(EmuCfg<NP, STAGE>::NT, emu_min_blocks(NP, STAG
   __syncthreads();
 
   // ---- phase 4: assemble, convert to FP64, scatter ----
-  float dps = 0.f, dpc = 0.f;  // (u, y) of this column, double-float
   const int64_t plane = P.gxs * P.gys;
   const bool ij_interior = (a > 0) && (a < N) && (b > 0) && (b < N) && !P.glo;
   const double unscale = exp2i(-shift);  // undoes the element's scaling of u (exact)
-#pragma unroll
-  for (int k = 0; k < NP; ++k) {
-    const int q = k * PS + b * RS + a;
-    float s = yt[k].x, c = yt[k].y;
-    dadd(s, c, sr[q]);
-    dadd(s, c, ss[q]);
-    if (P.wJa && active) {
-      const int64_t o = e * 2 * NP3 + t2 + NP2 * k;
-      dacc(s, c, P.wJa[o], P.wJa[o + NP3], uc[k]);
-    }
-    const float2 yk = dnorm(s, c);
-    if ((dirbits >> k) & 1u) continue;
-    if (DOT && P.partials) dacc(dps, dpc, uc[k].x, uc[k].y, yk);
-    int64_t g;
+  auto node_of = [&](int k) -> int64_t {
     if constexpr (BOXM) {
-      g = gbase + k * plane;
+      return gbase + k * plane;
     } else {
-      if (P.glo) {
-        g = P.glo[e * NP3 + t2 + NP2 * k];
-      } else {
-        const int64_t ex = e % P.sx, ey = (e / P.sx) % P.sy, ez = e / ((int64_t)P.sx * P.sy);
-        g = (ex * N + a) + P.gxs * ((ey * N + b) + P.gys * (ez * N + k));
-      }
+      if (P.glo) return P.glo[e * NP3 + t2 + NP2 * k];
+      const int64_t ex = e % P.sx, ey = (e / P.sx) % P.sy, ez = e / ((int64_t)P.sx * P.sy);
+      return (ex * N + a) + P.gxs * ((ey * N + b) + P.gys * (ez * N + k));
     }
-    const double yd = df_to_f64(yk) * unscale;
-    if (ij_interior && k > 0 && k < N)
-      P.y[g] = yd;
-    else
-      atomicAdd(P.y + g, yd);
-  }
-
-  if (DOT && P.partials) {
-    // (u, y) of the scaled values carries the element's scale twice
-    const double bs = block_sum<NT>(df_to_f64(dnorm(dps, dpc)) * unscale * unscale, s_red);
-    double pAp;
-    if (publish_partial_2level<NT>(bs, P.partials, P.gpartials, P.gtickets, &P.scal->counter[0], s_red, s_flag,
-                                   &pAp)) {
-      if (tid == 0) {
-        SemScalars *S = P.scal;
-        S->pAp = pAp;
-        if (!(pAp > 0.0) || !isfinite(pAp) || !isfinite(S->rz)) {
-          S->breakdown = 1;
-          S->alpha = 0.0;
-        } else {
-          S->alpha = S->rz / pAp;
-        }
-        S->counter[0] = 0;
+  };
+  if constexpr (DOT) {
+    // (u, y) of this column in double-float; the scaled values carry the element's scale twice.  One
+    // warp adds the block's values and publishes them before its scatter.
+    float dps = 0.f, dpc = 0.f;
+#pragma unroll
+    for (int k = 0; k < NP; ++k) {
+      const int q = k * PS + b * RS + a;
+      float s = yt[k].x, c = yt[k].y;
+      dadd(s, c, sr[q]);
+      dadd(s, c, ss[q]);
+      if (P.wJa && active) {
+        const int64_t o = e * 2 * NP3 + t2 + NP2 * k;
+        dacc(s, c, P.wJa[o], P.wJa[o + NP3], uc[k]);
       }
+      yt[k] = dnorm(s, c);
+      if (!((dirbits >> k) & 1u)) dacc(dps, dpc, uc[k].x, uc[k].y, yt[k]);
+    }
+    s_red[tid] = df_to_f64(dnorm(dps, dpc)) * unscale * unscale;
+    __syncthreads();
+    if (tid < 32) {
+      double pAp;
+      if (warp_publish_2level(warp_sum(s_red, NT), P.partials, P.gpartials, P.gtickets, &P.scal->counter[0], &pAp) &&
+          tid == 0)
+        cg_set_alpha(P.scal, pAp);
+    }
+#pragma unroll
+    for (int k = 0; k < NP; ++k) {
+      if ((dirbits >> k) & 1u) continue;
+      const double yd = df_to_f64(yt[k]) * unscale;
+      if (ij_interior && k > 0 && k < N)
+        P.y[node_of(k)] = yd;
+      else
+        atomicAdd(P.y + node_of(k), yd);
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < NP; ++k) {
+      const int q = k * PS + b * RS + a;
+      float s = yt[k].x, c = yt[k].y;
+      dadd(s, c, sr[q]);
+      dadd(s, c, ss[q]);
+      if (P.wJa && active) {
+        const int64_t o = e * 2 * NP3 + t2 + NP2 * k;
+        dacc(s, c, P.wJa[o], P.wJa[o + NP3], uc[k]);
+      }
+      const float2 yk = dnorm(s, c);
+      if ((dirbits >> k) & 1u) continue;
+      const int64_t g = node_of(k);
+      const double yd = df_to_f64(yk) * unscale;
+      if (ij_interior && k > 0 && k < N)
+        P.y[g] = yd;
+      else
+        atomicAdd(P.y + g, yd);
     }
   }
 }
 
 template <int NP, bool BOXM, bool STAGE, bool DOT>
 sem_status launch_k(const EmuParams<NP> &p, cudaStream_t s) {
-  using C = EmuCfg<NP, STAGE>;
+  using C = EmuCfg<NP, STAGE, DOT>;
   const unsigned grid = (unsigned)((p.E + C::EB - 1) / C::EB);
   if (p.partials && grid > SEM_MAX_PARTIALS) return sem_fail(SEM_ERR_INVALID, "too many elements for fused dot");
   static std::atomic<unsigned long long> attr_done;

@@ -70,50 +70,118 @@ __global__ void __launch_bounds__(VT) k_cg_init(int64_t G, const double *b, doub
   }
 }
 
+// The two vector kernels of a CG iteration walk the vectors 16 bytes at a time: UT threads per block,
+// at most two blocks per SM, each thread with the loads of two steps in flight.
+constexpr int UT = 512, UBLOCKS = 152 * 2;
+
 template <typename T>
-__global__ void __launch_bounds__(VT) k_cg_update(int64_t G, T *x, const T *p, T *r, const T *Ap, const T *dinv,
-                                                  SemScalars *S, double *partials) {
-  __shared__ double s_red[32];
-  __shared__ int s_flag;
+struct alignas(16) Vec16 {
+  static constexpr int N = 16 / sizeof(T);
+  T v[N];
+};
+
+// VEC: x too starts on a 16-byte boundary (the other vectors always do: they lie in the workspace).
+// Bound by HBM (7 words per node), or by the sums' latency while the vectors stay in L2: per-thread
+// sums in the vector precision, one per vector component (G / 622k entries each in FP32; FP64
+// arithmetic per entry would cost more than the traffic), one warp per quantity then adds the block's
+// in FP64.  1.4e6 nodes,
+// FP32: 22 us with 1216 blocks and a butterfly on every warp of each, 13.7 us now (caches
+// flushed before both).
+template <typename T, bool VEC>
+__global__ void __launch_bounds__(UT, 2) k_cg_update(int64_t G, T *__restrict__ x, const T *__restrict__ p,
+                                                     T *__restrict__ r, const T *__restrict__ Ap,
+                                                     const T *__restrict__ dinv, SemScalars *S, double *partials) {
+  constexpr int N = VEC ? Vec16<T>::N : 1;
+  struct alignas(N * sizeof(T)) V {
+    T v[N];
+  };
+  __shared__ T s_part[2][UT];
+  __shared__ double s_tot[2];
+  __shared__ int s_last;
   if (S->converged || S->breakdown) return;
   const T alpha = (T)S->alpha;
-  // per-thread partial sums in the vector precision (a thread sees about G / 311k entries; FP64
-  // arithmetic per entry would cost more than the traffic on GB300), widened for the block sum
-  T rz = T(0), rr = T(0);
-  for (int64_t g = (int64_t)blockIdx.x * VT + threadIdx.x; g < G; g += (int64_t)gridDim.x * VT) {
-    x[g] += alpha * p[g];
-    const T rg = r[g] - alpha * Ap[g];
-    r[g] = rg;
-    const T z = rg * dinv[g];
-    rz += rg * z;
-    rr += rg * rg;
+  const int tid = threadIdx.x, warp = tid >> 5;
+  T rz[N] = {}, rr[N] = {};
+  auto node = [&](int k, T &xv, T pv, T &rv, T av, T dv) {
+    xv += alpha * pv;
+    rv -= alpha * av;
+    const T z = rv * dv;
+    rz[k] += rv * z;
+    rr[k] += rv * rv;
+  };
+  const int64_t nv = G / N;
+#pragma unroll 2
+  for (int64_t g = (int64_t)blockIdx.x * UT + tid; g < nv; g += (int64_t)gridDim.x * UT) {
+    V xv = reinterpret_cast<V *>(x)[g], rv = reinterpret_cast<V *>(r)[g];
+    const V pv = reinterpret_cast<const V *>(p)[g], av = reinterpret_cast<const V *>(Ap)[g],
+            dv = reinterpret_cast<const V *>(dinv)[g];
+#pragma unroll
+    for (int k = 0; k < N; ++k) node(k, xv.v[k], pv.v[k], rv.v[k], av.v[k], dv.v[k]);
+    reinterpret_cast<V *>(x)[g] = xv;
+    reinterpret_cast<V *>(r)[g] = rv;
   }
-  const double a = block_sum<VT>((double)rz, s_red), c = block_sum<VT>((double)rr, s_red);
-  if (threadIdx.x == 0) {
-    partials[blockIdx.x] = a;
-    partials[gridDim.x + blockIdx.x] = c;
+  if (blockIdx.x == 0 && tid < (int)(G - nv * N)) {
+    const int64_t g = nv * N + tid;
+    node(0, x[g], p[g], r[g], Ap[g], dinv[g]);
   }
-  if (publish_partial<VT>(0.0, partials + 2 * gridDim.x, &S->counter[2], s_red, &s_flag)) {
-    const double RZ = final_sum<VT>(partials, gridDim.x, s_red);
-    const double RR = final_sum<VT>(partials + gridDim.x, gridDim.x, s_red);
-    if (threadIdx.x == 0) {
-      S->beta = RZ / S->rz;
-      S->rz = RZ;
-      S->rr = RR;
-      S->iter += 1;
-      if (!isfinite(RR) || !isfinite(RZ)) S->breakdown = 1;
-      if (RR <= S->tol2) S->converged = 1;
-      S->counter[2] = 0;
-    }
+#pragma unroll
+  for (int w = N / 2; w > 0; w /= 2)
+#pragma unroll
+    for (int k = 0; k < w; ++k) rz[k] += rz[k + w], rr[k] += rr[k + w];
+  s_part[0][tid] = rz[0];
+  s_part[1][tid] = rr[0];
+  __syncthreads();
+  if (warp < 2) {
+    const double v = warp_sum(s_part[warp], UT);
+    if ((tid & 31) == 0) partials[warp * gridDim.x + blockIdx.x] = v;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    __threadfence();
+    s_last = atomicAdd(&S->counter[2], 1u) == gridDim.x - 1u;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  if (warp < 2) {
+    const double v = warp_sum_partials(partials + warp * gridDim.x, gridDim.x);
+    if ((tid & 31) == 0) s_tot[warp] = v;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    const double RZ = s_tot[0], RR = s_tot[1];
+    S->beta = RZ / S->rz;
+    S->rz = RZ;
+    S->rr = RR;
+    S->iter += 1;
+    if (!isfinite(RR) || !isfinite(RZ)) S->breakdown = 1;
+    if (RR <= S->tol2) S->converged = 1;
+    S->counter[2] = 0;
   }
 }
 
 template <typename T>
-__global__ void __launch_bounds__(VT) k_cg_direction(int64_t G, T *p, const T *r, T *Ap, const T *dinv,
-                                                     const SemScalars *S) {
+__global__ void __launch_bounds__(UT, 2) k_cg_direction(int64_t G, T *__restrict__ p, const T *__restrict__ r,
+                                                        T *__restrict__ Ap, const T *__restrict__ dinv,
+                                                        const SemScalars *S) {
   if (S->converged || S->breakdown) return;
   const T beta = (T)S->beta;
-  for (int64_t g = (int64_t)blockIdx.x * VT + threadIdx.x; g < G; g += (int64_t)gridDim.x * VT) {
+  using V = Vec16<T>;
+  const int64_t nv = G / V::N;
+#pragma unroll 2
+  for (int64_t g = (int64_t)blockIdx.x * UT + threadIdx.x; g < nv; g += (int64_t)gridDim.x * UT) {
+    const V rv = reinterpret_cast<const V *>(r)[g], dv = reinterpret_cast<const V *>(dinv)[g];
+    V pv = reinterpret_cast<V *>(p)[g], zero;
+#pragma unroll
+    for (int k = 0; k < V::N; ++k) {
+      pv.v[k] = rv.v[k] * dv.v[k] + beta * pv.v[k];
+      zero.v[k] = T(0);
+    }
+    reinterpret_cast<V *>(p)[g] = pv;
+    reinterpret_cast<V *>(Ap)[g] = zero;
+  }
+  if (blockIdx.x == 0 && threadIdx.x < G - nv * V::N) {
+    const int64_t g = nv * V::N + threadIdx.x;
     p[g] = r[g] * dinv[g] + beta * p[g];
     Ap[g] = T(0);
   }
@@ -276,6 +344,12 @@ inline unsigned vgrid(int64_t G) {
   return (unsigned)std::max<int64_t>(1, std::min<int64_t>(VBLOCKS, need));
 }
 
+// grid of the CG vector kernels: one vector of `per` nodes per thread, at most UBLOCKS blocks
+inline unsigned ugrid(int64_t G, int per) {
+  const int64_t need = (G + (int64_t)per * UT - 1) / ((int64_t)per * UT);
+  return (unsigned)std::max<int64_t>(1, std::min<int64_t>(UBLOCKS, need));
+}
+
 // Copies the solver scalars to the host (synchronising the stream).  A bounded device wait that
 // gave up since the solve started (an apply left its output incomplete) ends the solve with
 // SEM_ERR_TIMEOUT; the flag and the reduction tickets are cleared for later calls.
@@ -311,53 +385,68 @@ struct History {
   }
 };
 
+// Captures what `body` launches on st and makes it an executable graph (*exec).
+template <typename F>
+sem_status capture_graph(cudaStream_t st, cudaGraphExec_t *exec, F body) {
+  cudaGraph_t g = nullptr;
+  sem_status s = SEM_OK;
+  cudaError_t ce = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
+  if (ce == cudaSuccess) {
+    s = body(st);
+    ce = cudaStreamEndCapture(st, &g);
+  }
+  if (s == SEM_OK && ce != cudaSuccess)
+    s = sem_fail(SEM_ERR_CUDA, std::string("graph capture: ") + cudaGetErrorString(ce));
+  if (s == SEM_OK) {
+    ce = cudaGraphInstantiate(exec, g, 0);
+    if (ce != cudaSuccess) s = sem_fail(SEM_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(ce));
+  }
+  if (g) cudaGraphDestroy(g);
+  return s;
+}
+
 // One block of `count` CG iterations on type T.
 template <typename T>
 sem_status cg_block(sem_handle *h, int prec, int count, T *x, T *p, T *r, T *Ap, const T *dinv, cudaStream_t st) {
   for (int it = 0; it < count; ++it) {
     sem_status s = sem_launch_apply(h, (sem_prec)prec, p, Ap, h->partials, nullptr, nullptr, st);
     if (s != SEM_OK) return s;
-    k_cg_update<T><<<vgrid(h->G), VT, 0, st>>>(h->G, x, p, r, Ap, dinv, h->scal, h->partials);
-    k_cg_direction<T><<<vgrid(h->G), VT, 0, st>>>(h->G, p, r, Ap, dinv, h->scal);
+    const unsigned grid = ugrid(h->G, Vec16<T>::N);
+    if (reinterpret_cast<uintptr_t>(x) % 16 == 0)
+      k_cg_update<T, true><<<grid, UT, 0, st>>>(h->G, x, p, r, Ap, dinv, h->scal, h->partials);
+    else
+      k_cg_update<T, false><<<ugrid(h->G, 1), UT, 0, st>>>(h->G, x, p, r, Ap, dinv, h->scal, h->partials);
+    k_cg_direction<T><<<grid, UT, 0, st>>>(h->G, p, r, Ap, dinv, h->scal);
   }
   SEM_CUDA_TRY(cudaGetLastError());
   return SEM_OK;
 }
 
 // Runs CG from the state set up by k_cg_init until convergence, breakdown or max_it.
-// hist (may be null) gets (it0 + iterations, sqrt(rr / bb)) at each host check.
+// exec: the graph of check_every iterations, captured at its first use and kept by the caller for its
+// later calls with the same vectors.  hist (may be null) gets (it0 + iterations, sqrt(rr / bb)) at
+// each host check.
 template <typename T>
 sem_status cg_run(sem_handle *h, int prec, const sem_pcg_opts *o, T *x, T *p, T *r, T *Ap, const T *dinv,
-                  cudaStream_t st, int *iters, double *rr_out, int budget, History *hist = nullptr, int it0 = 0,
-                  double bb = 0.0) {
+                  cudaStream_t st, cudaGraphExec_t *exec, int *iters, double *rr_out, int budget,
+                  History *hist = nullptr, int it0 = 0, double bb = 0.0) {
   SemScalars hs;
   sem_status s = read_scalars(h, &hs, st);
   if (s != SEM_OK) return s;
   if (hist && bb > 0) hist->add(it0 + hs.iter, sqrt(hs.rr / bb));
   const int every = std::max(1, o->check_every);
-  cudaGraphExec_t exec = nullptr;
-  bool graph = o->use_graph && st != nullptr;
   while (!hs.converged && !hs.breakdown && hs.iter < budget) {
     const int count = std::min(every, budget - hs.iter);
-    if (graph && count == every) {
-      if (!exec) {
-        cudaGraph_t g;
-        SEM_CUDA_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-        sem_status cs = cg_block<T>(h, prec, count, x, p, r, Ap, dinv, st);
-        cudaError_t ce = cudaStreamEndCapture(st, &g);
-        if (cs != SEM_OK) {
-          if (ce == cudaSuccess) cudaGraphDestroy(g);
-          return cs;
-        }
-        if (ce != cudaSuccess) return sem_fail(SEM_ERR_CUDA, std::string("graph capture: ") + cudaGetErrorString(ce));
-        ce = cudaGraphInstantiate(&exec, g, 0);
-        cudaGraphDestroy(g);
-        if (ce != cudaSuccess) return sem_fail(SEM_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(ce));
+    if (o->use_graph && st && count == every) {
+      if (!*exec) {
+        s = capture_graph(st, exec,
+                          [&](cudaStream_t cap) { return cg_block<T>(h, prec, count, x, p, r, Ap, dinv, cap); });
+        if (s != SEM_OK) break;
       }
-      cudaError_t ce = cudaGraphLaunch(exec, st);
+      const cudaError_t ce = cudaGraphLaunch(*exec, st);
       if (ce != cudaSuccess) {
-        cudaGraphExecDestroy(exec);
-        return sem_fail(SEM_ERR_CUDA, std::string("graph launch: ") + cudaGetErrorString(ce));
+        s = sem_fail(SEM_ERR_CUDA, std::string("graph launch: ") + cudaGetErrorString(ce));
+        break;
       }
     } else {
       s = cg_block<T>(h, prec, count, x, p, r, Ap, dinv, st);
@@ -367,7 +456,6 @@ sem_status cg_run(sem_handle *h, int prec, const sem_pcg_opts *o, T *x, T *p, T 
     if (s != SEM_OK) break;
     if (hist && bb > 0) hist->add(it0 + hs.iter, sqrt(hs.rr / bb));
   }
-  if (exec) cudaGraphExecDestroy(exec);
   if (s != SEM_OK) return s;
   *iters = hs.iter;
   *rr_out = hs.rr;
@@ -425,6 +513,12 @@ extern "C" sem_status sem_pcg(sem_handle *h, const double *d_b, double *d_x, con
   const int64_t G = h->G;
   sem_status s = SEM_OK;
   SemScalars hs;
+  struct Exec {  // the solve's step graph, released on every way out
+    cudaGraphExec_t e = nullptr;
+    ~Exec() {
+      if (e) cudaGraphExecDestroy(e);
+    }
+  } exec;
   SEM_CUDA_TRY(cudaMemsetAsync(h->scal, 0, sizeof(SemScalars), st));
 
   if (o->mode == SEM_SOLVE_FP64) {
@@ -446,7 +540,7 @@ extern "C" sem_status sem_pcg(sem_handle *h, const double *d_b, double *d_x, con
       const double bb = hs.bb;
       int iters = 0;
       double rr = 0.0;
-      s = cg_run<double>(h, prec64, o, d_x, h->p64, h->r64, h->Ap64, h->dinv64, st, &iters, &rr,
+      s = cg_run<double>(h, prec64, o, d_x, h->p64, h->r64, h->Ap64, h->dinv64, st, &exec.e, &iters, &rr,
                          std::max(1, o->max_it - total), &hist, total, bb);
       total += iters;
       res->recursive_relres = bb > 0 ? sqrt(rr / bb) : 0.0;
@@ -502,7 +596,7 @@ extern "C" sem_status sem_pcg(sem_handle *h, const double *d_b, double *d_x, con
                                                 h->dinv32, h->scal, h->partials, inner * inner);
       int iters = 0;
       double rr = 0.0;
-      s = cg_run<float>(h, inner_prec, o, h->x32, h->p32, h->r32, h->Ap32, h->dinv32, st, &iters, &rr,
+      s = cg_run<float>(h, inner_prec, o, h->x32, h->p32, h->r32, h->Ap32, h->dinv32, st, &exec.e, &iters, &rr,
                         std::max(1, o->max_it - total));
       total += iters;
       if (s == SEM_ERR_NOCONV) s = SEM_OK;  // a partial inner solve still improves x
@@ -533,7 +627,6 @@ extern "C" sem_status sem_pcg(sem_handle *h, const double *d_b, double *d_x, con
     // blocks of check_every iterations, decided on the device (fallback, beta, alpha, convergence),
     // replayed as one CUDA graph; the host reads the scalars once per block
     const int every = std::max(1, o->check_every);
-    cudaGraphExec_t exec = nullptr;
     const bool graph = o->use_graph && st != nullptr;
     bool eager_done = false;  // one eager iteration first: attributes and tables are set up before capture
     // When the recursive residual meets the tolerance but the FP64-accurate true residual does
@@ -544,22 +637,11 @@ extern "C" sem_status sem_pcg(sem_handle *h, const double *d_b, double *d_x, con
       while (s == SEM_OK && !hs.converged && !hs.breakdown && hs.iter < o->max_it) {
         const int count = std::min(every, o->max_it - hs.iter);
         if (graph && eager_done && count == every) {
-          if (!exec) {
-            cudaGraph_t g;
-            SEM_CUDA_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-            sem_status cs = fcg_block(h, prec64, count, d_x, st);
-            cudaError_t ce = cudaStreamEndCapture(st, &g);
-            if (cs != SEM_OK) {
-              if (ce == cudaSuccess) cudaGraphDestroy(g);
-              return ret(cs);
-            }
-            if (ce != cudaSuccess) return ret(sem_fail(SEM_ERR_CUDA, std::string("graph capture: ") + cudaGetErrorString(ce)));
-            ce = cudaGraphInstantiate(&exec, g, 0);
-            cudaGraphDestroy(g);
-            if (ce != cudaSuccess)
-              return ret(sem_fail(SEM_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(ce)));
+          if (!exec.e) {
+            s = capture_graph(st, &exec.e, [&](cudaStream_t cap) { return fcg_block(h, prec64, count, d_x, cap); });
+            if (s != SEM_OK) break;
           }
-          const cudaError_t ce = cudaGraphLaunch(exec, st);
+          const cudaError_t ce = cudaGraphLaunch(exec.e, st);
           if (ce != cudaSuccess) s = sem_fail(SEM_ERR_CUDA, std::string("graph launch: ") + cudaGetErrorString(ce));
         } else {
           s = fcg_block(h, prec64, graph && !eager_done ? 1 : count, d_x, st);
@@ -580,7 +662,6 @@ extern "C" sem_status sem_pcg(sem_handle *h, const double *d_b, double *d_x, con
       hs.restart_iter = hs.iter;
       SEM_CUDA_TRY(cudaMemcpyAsync(h->scal, &hs, sizeof(SemScalars), cudaMemcpyHostToDevice, st));
     }
-    if (exec) cudaGraphExecDestroy(exec);
     if (s == SEM_OK && hs.breakdown) s = sem_fail(SEM_ERR_BREAKDOWN, "flexible CG breakdown");
     const int fallbacks = hs.nfallback;
     if (s == SEM_OK && !hs.converged) s = sem_fail(SEM_ERR_NOCONV, "flexible CG: max_it reached");
