@@ -38,16 +38,20 @@ struct DConst {
   T v[NP * NP];  // D[i][m] at v[i * NP + m]
   // Even-odd form of D (index 0) and D^T (index 1), both centro-antisymmetric
   // (M[N-i][N-m] = -M[i][m]): for i, m < H = NP/2, A = (M[i][m] + M[i][N-m]) / 2,
-  // B = (M[i][m] - M[i][N-m]) / 2; for odd NP the middle column C[i] = M[i][H] and the middle
-  // row R[m] = M[H][m].
-  T A[2][(NP / 2) * (NP / 2)], B[2][(NP / 2) * (NP / 2)], C[2][NP / 2 + 1], R[2][NP / 2 + 1];
+  // B = (M[i][m] - M[i][N-m]) / 2, stored as pairs (B, A); for odd NP the middle column
+  // C[i] = M[i][H] and the middle row R[m] = M[H][m].
+  struct alignas(2 * sizeof(T)) Pair {
+    T b, a;
+  };
+  Pair BA[2][(NP / 2) * (NP / 2)];
+  T C[2][NP / 2 + 1], R[2][NP / 2 + 1];
 };
 
 // y = M v for a centro-antisymmetric NP x NP matrix M given in even-odd form (DConst, index t):
 // with e_m = v_m + v_{N-m}, o_m = v_m - v_{N-m} (m < H), P_i = sum_m B_im o_m and
 // Q_i = sum_m A_im e_m (+ C_i v_H for odd NP), y_i = P_i + Q_i and y_{N-i} = P_i - Q_i; the middle
 // output of odd NP is sum_m R_m o_m (M[H][H] = 0).  2 H^2 products instead of NP^2.
-template <int NP, typename T>
+template <int NP, typename T, bool PK>
 __device__ __forceinline__ void line_eo(const DConst<NP, T> &D, int t, const T (&v)[NP], T (&y)[NP]) {
   constexpr int H = NP / 2, N = NP - 1;
   T e[H], o[H];
@@ -59,10 +63,21 @@ __device__ __forceinline__ void line_eo(const DConst<NP, T> &D, int t, const T (
 #pragma unroll
   for (int i = 0; i < H; ++i) {
     T P = T(0), Q = T(0);
+    if constexpr (PK) {
+      // P and Q together in packed FMAs (the scalar rate at half the issue slots, same rounding)
+      float2 PQ = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int m = 0; m < H; ++m) {
-      P += D.B[t][i * H + m] * o[m];
-      Q += D.A[t][i * H + m] * e[m];
+      for (int m = 0; m < H; ++m) {
+        const auto c = D.BA[t][i * H + m];
+        PQ = __ffma2_rn(make_float2(c.b, c.a), make_float2(o[m], e[m]), PQ);
+      }
+      P = PQ.x, Q = PQ.y;
+    } else {
+#pragma unroll
+      for (int m = 0; m < H; ++m) {
+        P += D.BA[t][i * H + m].b * o[m];
+        Q += D.BA[t][i * H + m].a * e[m];
+      }
     }
     if constexpr (NP % 2 == 1) Q += D.C[t][i] * v[H];
     y[i] = P + Q;
@@ -79,7 +94,7 @@ __device__ __forceinline__ void line_eo(const DConst<NP, T> &D, int t, const T (
 // y = M v with M = D (t = 0) or D^T (t = 1): the even-odd form, except for FP32 above NP = 12,
 // where the plain product measured faster (register pressure of the split: 64 -> 50 GDOF/s at
 // N = 15, against +40% at N = 11 and +25% for FP64)
-template <int NP, typename T>
+template <int NP, typename T, bool PK>
 __device__ __forceinline__ void line_apply(const DConst<NP, T> &D, int t, const T (&v)[NP], T (&y)[NP]) {
   if constexpr (sizeof(T) == 4 && NP > 12) {
 #pragma unroll
@@ -90,7 +105,7 @@ __device__ __forceinline__ void line_apply(const DConst<NP, T> &D, int t, const 
       y[i] = acc;
     }
   } else {
-    line_eo<NP, T>(D, t, v, y);
+    line_eo<NP, T, PK && sizeof(T) == 4>(D, t, v, y);
   }
 }
 
@@ -103,8 +118,8 @@ __host__ void fill_dconst(DConst<NP, T> &D, const double *Dd) {
     auto M = [&](int i, int m) { return t == 0 ? Dd[i * NP + m] : Dd[m * NP + i]; };
     for (int i = 0; i < H; ++i)
       for (int m = 0; m < H; ++m) {
-        D.A[t][i * H + m] = (T)(0.5 * (M(i, m) + M(i, N - m)));
-        D.B[t][i * H + m] = (T)(0.5 * (M(i, m) - M(i, N - m)));
+        D.BA[t][i * H + m].a = (T)(0.5 * (M(i, m) + M(i, N - m)));
+        D.BA[t][i * H + m].b = (T)(0.5 * (M(i, m) - M(i, N - m)));
       }
     for (int i = 0; i <= H; ++i) {
       D.C[t][i] = (NP % 2 == 1 && i < H) ? (T)M(i, H) : T(0);
@@ -288,6 +303,24 @@ __host__ __device__ constexpr bool apply_loop_dirs(int NP) {
   return !is_otf<TG>() && sizeof(T) == 4 && (NP == 14 || NP == 15);
 }
 
+// FP32 with stored factors read directly: a thread's 6 NP factors are asked for before anything else
+// and held in registers (small orders only), so that their latency runs beside the gather and the
+// gradients instead of after them.
+// GDOF/s at 8e6 nodes, without / with: N = 3 105 / 121, 4 102 / 111, 5 99 / 111 (BF16 factors are
+// staged instead there, see apply_auto_variant).
+template <typename T, typename TG, bool STAGE>
+__host__ __device__ constexpr bool apply_prefetch(int NP) {
+  return !STAGE && std::is_same<T, float>::value && std::is_same<TG, float>::value && NP <= 6;
+}
+
+// Packed line products (line_eo).  GDOF/s at 8e6 nodes, scalar / packed: FP32 factors N = 3 121 / 116, 5
+// 111 / 105, 7 120 / 122, 10 113 / 115; BF16 7 138 / 144, 8 133 / 151, 9 125 / 143; on the fly 4 118 / 129,
+// 5 114 / 126, 7 149 / 155, 9 125 / 118, 10 145 / 151.
+template <typename T, typename TG>
+__host__ __device__ constexpr bool apply_packed(int NP) {
+  return sizeof(T) == 4 && (is_otf<TG>() ? NP != 10 : sizeof(TG) == 2 || NP >= 7);
+}
+
 // TG: storage type of the factors (T, or BF16 with T = float: half the factor traffic)
 template <int NP, typename T, int EB_, bool STAGE, bool BOXM, typename TG = T>
 __global__ void __launch_bounds__(ApplyCfg<NP, EB_>::NT, apply_min_blocks<T>(NP, EB_))
@@ -297,6 +330,7 @@ __global__ void __launch_bounds__(ApplyCfg<NP, EB_>::NT, apply_min_blocks<T>(NP,
                 BUF = C::BUF, GS = factor_stride<NP, TG>();
   extern __shared__ __align__(128) unsigned char smem_raw[];
   constexpr size_t RED_OFF = apply_red_off<NP, T, EB_, STAGE, TG>();
+  constexpr bool PK = apply_packed<T, TG>(NP);
   static_assert(RED_OFF % 16 == 0 && ((STAGE ? EB * GS : 0) * sizeof(TG)) % 16 == 0, "shared-memory alignment");
   TG *sG = reinterpret_cast<TG *>(smem_raw);  // TMA destination: 16-byte aligned at offset 0
   T *sbuf = reinterpret_cast<T *>(smem_raw + (STAGE ? EB * GS * sizeof(TG) : 0));
@@ -361,6 +395,13 @@ __global__ void __launch_bounds__(ApplyCfg<NP, EB_>::NT, apply_min_blocks<T>(NP,
       const bool skip = !active || (B.done && *B.done);
       if (__syncthreads_and(skip)) return;  // every element of this block is finished
     }
+  }
+  constexpr bool PREF = apply_prefetch<T, TG, STAGE>(NP);
+  TG gpre[PREF ? 6 * NP : 1];
+  if constexpr (PREF) {
+    const TG *Ge = c_Gf + (active ? el : 0) * P.gs + t2;
+#pragma unroll
+    for (int q = 0; q < 6 * NP; ++q) gpre[q] = active ? Ge[q / NP * NP3 + q % NP * NP2] : TG(0.f);
   }
   if constexpr (BOXM) {
     const int64_t plane = c_gxs * c_gys;
@@ -430,7 +471,7 @@ __global__ void __launch_bounds__(ApplyCfg<NP, EB_>::NT, apply_min_blocks<T>(NP,
       T row[NP], out[NP];
 #pragma unroll
       for (int m = 0; m < NP; ++m) row[m] = su[ib + m * is];
-      line_apply<NP, T>(P.D, 0, row, out);
+      line_apply<NP, T, PK>(P.D, 0, row, out);
       if (dir == 2) {
 #pragma unroll
         for (int k = 0; k < NP; ++k) wt[k] = out[k];
@@ -441,16 +482,16 @@ __global__ void __launch_bounds__(ApplyCfg<NP, EB_>::NT, apply_min_blocks<T>(NP,
       }
     }
   } else {
-    line_apply<NP, T>(P.D, 0, uc, wt);
+    line_apply<NP, T, PK>(P.D, 0, uc, wt);
     T row[NP], out[NP];
 #pragma unroll
     for (int m = 0; m < NP; ++m) row[m] = su[b * PS + a * RS + m];  // u(m, j=a, k=b)
-    line_apply<NP, T>(P.D, 0, row, out);
+    line_apply<NP, T, PK>(P.D, 0, row, out);
 #pragma unroll
     for (int i = 0; i < NP; ++i) sr[b * PS + a * RS + i] = out[i];
 #pragma unroll
     for (int m = 0; m < NP; ++m) row[m] = su[b * PS + m * RS + a];  // u(i=a, m, k=b)
-    line_apply<NP, T>(P.D, 0, row, out);
+    line_apply<NP, T, PK>(P.D, 0, row, out);
 #pragma unroll
     for (int j = 0; j < NP; ++j) ss[b * PS + j * RS + a] = out[j];
   }
@@ -503,7 +544,14 @@ __global__ void __launch_bounds__(ApplyCfg<NP, EB_>::NT, apply_min_blocks<T>(NP,
       const int q = k * PS + b * RS + a;
       const int o = k * NP2;
       T g0 = T(0), g1 = T(0), g2 = T(0), g3 = T(0), g4 = T(0), g5 = T(0);
-      if (STAGE || active) {
+      if constexpr (PREF) {
+        g0 = widen<T, TG>(gpre[k]);
+        g1 = widen<T, TG>(gpre[NP + k]);
+        g2 = widen<T, TG>(gpre[2 * NP + k]);
+        g3 = widen<T, TG>(gpre[3 * NP + k]);
+        g4 = widen<T, TG>(gpre[4 * NP + k]);
+        g5 = widen<T, TG>(gpre[5 * NP + k]);
+      } else if (STAGE || active) {
         g0 = widen<T, TG>(Ge[0 * NP3 + o]);
         g1 = widen<T, TG>(Ge[1 * NP3 + o]);
         g2 = widen<T, TG>(Ge[2 * NP3 + o]);
@@ -530,7 +578,7 @@ __global__ void __launch_bounds__(ApplyCfg<NP, EB_>::NT, apply_min_blocks<T>(NP,
       T row[NP], out[NP];
 #pragma unroll
       for (int m = 0; m < NP; ++m) row[m] = dir == 2 ? wt[m] : buf[ib + m * is];
-      line_apply<NP, T>(P.D, 1, row, out);
+      line_apply<NP, T, PK>(P.D, 1, row, out);
       if (dir == 2) {
 #pragma unroll
         for (int k = 0; k < NP; ++k) yc[k] = out[k];
@@ -540,19 +588,19 @@ __global__ void __launch_bounds__(ApplyCfg<NP, EB_>::NT, apply_min_blocks<T>(NP,
       }
     }
   } else {
-    line_apply<NP, T>(P.D, 1, wt, yc);
+    line_apply<NP, T, PK>(P.D, 1, wt, yc);
     __syncthreads();
 
     // ---- phase 3: transposed r and s contractions ----
     T row[NP], out[NP];
 #pragma unroll
     for (int m = 0; m < NP; ++m) row[m] = sr[b * PS + a * RS + m];  // w_r(m, j=a, k=b)
-    line_apply<NP, T>(P.D, 1, row, out);
+    line_apply<NP, T, PK>(P.D, 1, row, out);
 #pragma unroll
     for (int i = 0; i < NP; ++i) sr[b * PS + a * RS + i] = out[i];
 #pragma unroll
     for (int m = 0; m < NP; ++m) row[m] = ss[b * PS + m * RS + a];  // w_s(i=a, m, k=b)
-    line_apply<NP, T>(P.D, 1, row, out);
+    line_apply<NP, T, PK>(P.D, 1, row, out);
 #pragma unroll
     for (int j = 0; j < NP; ++j) ss[b * PS + j * RS + a] = out[j];
   }
@@ -676,17 +724,24 @@ __host__ __device__ constexpr size_t pipe_smem();
 //      (structured boxes, when two factor blocks fit; otherwise variant 0)
 #define SEM_APPLY_VARIANTS 5
 
-// Variant chosen when the handle asks for automatic selection (-1): measured on GB300 over the
-// 64^3-element box at N = 3..15 (FP32: factor staging pays from N = 7 on, direct reads win
-// below; FP64 is bound by its FMA pipe and indifferent; on-the-fly factors: one element per
-// block at N = 3 and N = 6, 7, the default tile elsewhere).
-__host__ __device__ constexpr int apply_auto_variant(int NP, bool fp32, bool otf = false) {
-  return otf ? ((NP == 4 || NP == 7 || NP == 8) ? 3 : 1) : !fp32 ? 1 : (NP <= 6 ? 1 : NP == 16 ? 2 : 0);
+// Variant chosen when the handle asks for automatic selection (-1), measured on GB300 (GDOF/s at 8e6
+// nodes, variants 0 / 1 / 3): FP32 N = 2 116 / 109 / 113, 3 108 / 121 / 111, 5 107 / 111 / 110, 6 110 / 93 /
+// 113, 7 122 / 100 / 116, 15 56 / 56 / 56 (the former choice there, 2: 49); BF16 N = 2 141 / 120 / 136, 3
+// 145 / 127 / 145, 5 130 / 108 / 114, 6 135 / 105 / 140, 7 144 / 106 / 139, 15 74 / 58 / 74; on the fly
+// (no factor block: 0 = 1) N = 3 139 / 139, 5 126 / 97, 6 120 / 116, 7 147 / 155 (variants 1 / 3).  FP64 is
+// bound by its FMA pipe and indifferent.
+template <typename T, typename TG>
+__host__ __device__ constexpr int apply_auto_variant(int NP) {
+  return is_otf<TG>() ? (NP == 4 || NP == 8 ? 3 : 1)
+         : sizeof(T) == 8 ? 1
+         : NP == 7 ? 3
+         : sizeof(TG) == 2 ? 0
+         : (NP == 3 || (NP > 6 && NP < 16)) ? 0 : 1;
 }
 
 template <int NP, typename T, typename TG = T>
 static sem_status launch_apply_np(const ApplyParams<T, NP> &p, int variant, cudaStream_t s) {
-  if (variant < 0) variant = apply_auto_variant(NP, sizeof(T) == 4, is_otf<TG>());
+  if (variant < 0) variant = apply_auto_variant<T, TG>(NP);
   constexpr int EB0 = apply_eb_default(NP);
   constexpr int EB2 = (EB0 * 2 * NP * NP <= 1024 &&
                        apply_smem<NP, T, EB0 * 2, false, TG>() <= SEM_MAX_SMEM_PER_BLOCK) ? EB0 * 2 : EB0;

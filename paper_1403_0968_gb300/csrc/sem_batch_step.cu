@@ -86,6 +86,7 @@ __device__ __forceinline__ void fused_apply_tile(const SlotParams &S, int64_t ti
                                                  double *pAp, unsigned char *smem) {
   constexpr int N = NP - 1, NP2 = NP * NP, NP3 = NP2 * NP, EB = fused_eb(NP), ES = fused_es(NP);
   constexpr int RS = NP | 1, PS = NP * RS, BUF = fused_buf(NP);
+  // scalar line products: at 64 registers per thread the packed ones spill (111 against 110 ms a solve)
   static_assert(EB >= 1 && ES * NP2 >= FT, "tile against the block");
   const DConst<NP, float> &D = tab_D<NP>();
   float *sbuf = reinterpret_cast<float *>(smem);
@@ -134,17 +135,17 @@ __device__ __forceinline__ void fused_apply_tile(const SlotParams &S, int64_t ti
 
   // ---- gradients: u_t along the thread's column, u_r and u_s through shared memory ----
   float wt[NP];  // u_t, then w_t
-  line_apply<NP, float>(D, 0, uc, wt);
+  line_apply<NP, float, false>(D, 0, uc, wt);
   {
     float row[NP], out[NP];
 #pragma unroll
     for (int m = 0; m < NP; ++m) row[m] = su[b * PS + a * RS + m];  // u(m, j = a, k = b)
-    line_apply<NP, float>(D, 0, row, out);
+    line_apply<NP, float, false>(D, 0, row, out);
 #pragma unroll
     for (int i = 0; i < NP; ++i) sr[b * PS + a * RS + i] = out[i];
 #pragma unroll
     for (int m = 0; m < NP; ++m) row[m] = su[b * PS + m * RS + a];  // u(i = a, m, k = b)
-    line_apply<NP, float>(D, 0, row, out);
+    line_apply<NP, float, false>(D, 0, row, out);
 #pragma unroll
     for (int j = 0; j < NP; ++j) ss[b * PS + j * RS + a] = out[j];
   }
@@ -174,7 +175,7 @@ __device__ __forceinline__ void fused_apply_tile(const SlotParams &S, int64_t ti
     }
   }
   float yc[NP];
-  line_apply<NP, float>(D, 1, wt, yc);
+  line_apply<NP, float, false>(D, 1, wt, yc);
   __syncthreads();
 
   // ---- transposed r and s contractions ----
@@ -182,12 +183,12 @@ __device__ __forceinline__ void fused_apply_tile(const SlotParams &S, int64_t ti
     float row[NP], out[NP];
 #pragma unroll
     for (int m = 0; m < NP; ++m) row[m] = sr[b * PS + a * RS + m];  // w_r(m, j = a, k = b)
-    line_apply<NP, float>(D, 1, row, out);
+    line_apply<NP, float, false>(D, 1, row, out);
 #pragma unroll
     for (int i = 0; i < NP; ++i) sr[b * PS + a * RS + i] = out[i];
 #pragma unroll
     for (int m = 0; m < NP; ++m) row[m] = ss[b * PS + m * RS + a];  // w_s(i = a, m, k = b)
-    line_apply<NP, float>(D, 1, row, out);
+    line_apply<NP, float, false>(D, 1, row, out);
 #pragma unroll
     for (int j = 0; j < NP; ++j) ss[b * PS + j * RS + a] = out[j];
   }
