@@ -385,16 +385,20 @@ struct History {
   }
 };
 
-// Captures what `body` launches on st and makes it an executable graph (*exec).
+// Captures what `body` launches and makes it an executable graph (*exec).  The legacy default stream
+// cannot be captured: its work is captured on a stream of its own and replayed on the default one.
 template <typename F>
 sem_status capture_graph(cudaStream_t st, cudaGraphExec_t *exec, F body) {
+  cudaStream_t cap = st;
+  if (!st) SEM_CUDA_TRY(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
   cudaGraph_t g = nullptr;
   sem_status s = SEM_OK;
-  cudaError_t ce = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
+  cudaError_t ce = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
   if (ce == cudaSuccess) {
-    s = body(st);
-    ce = cudaStreamEndCapture(st, &g);
+    s = body(cap);
+    ce = cudaStreamEndCapture(cap, &g);
   }
+  if (!st) cudaStreamDestroy(cap);
   if (s == SEM_OK && ce != cudaSuccess)
     s = sem_fail(SEM_ERR_CUDA, std::string("graph capture: ") + cudaGetErrorString(ce));
   if (s == SEM_OK) {
@@ -437,7 +441,7 @@ sem_status cg_run(sem_handle *h, int prec, const sem_pcg_opts *o, T *x, T *p, T 
   const int every = std::max(1, o->check_every);
   while (!hs.converged && !hs.breakdown && hs.iter < budget) {
     const int count = std::min(every, budget - hs.iter);
-    if (o->use_graph && st && count == every) {
+    if (o->use_graph && count == every) {
       if (!*exec) {
         s = capture_graph(st, exec,
                           [&](cudaStream_t cap) { return cg_block<T>(h, prec, count, x, p, r, Ap, dinv, cap); });
@@ -627,7 +631,7 @@ extern "C" sem_status sem_pcg(sem_handle *h, const double *d_b, double *d_x, con
     // blocks of check_every iterations, decided on the device (fallback, beta, alpha, convergence),
     // replayed as one CUDA graph; the host reads the scalars once per block
     const int every = std::max(1, o->check_every);
-    const bool graph = o->use_graph && st != nullptr;
+    const bool graph = o->use_graph;
     bool eager_done = false;  // one eager iteration first: attributes and tables are set up before capture
     // When the recursive residual meets the tolerance but the FP64-accurate true residual does
     // not (the recurrence drifts over many iterations with a changing preconditioner), the
