@@ -311,13 +311,13 @@ __device__ __forceinline__ void df_line(const EmuParams<NP> &P, const float2 (&v
 __host__ __device__ constexpr int emu_eb_staged(int NP) {
   return NP <= 2 ? 32 : NP == 3 ? 14 : NP == 4 ? 8 : NP == 5 ? 5 : NP == 6 ? 3 : NP <= 8 ? 2 : 1;
 }
-__host__ __device__ constexpr int emu_eb(int NP) {
-  return NP == 6 ? 7 : NP == 7 ? 5 : (NP == 9 || NP == 10) ? 3 : NP == 12 ? 2 : emu_eb_staged(NP);
+__host__ __device__ constexpr int emu_eb(int NP, bool small) {
+  return small ? emu_eb_staged(NP) : NP == 6 ? 7 : NP == 7 ? 5 : (NP == 9 || NP == 10) ? 3 : NP == 12 ? 2 : emu_eb_staged(NP);
 }
 
-template <int NP, bool STAGE, bool DOT>
+template <int NP, bool STAGE, bool DOT, bool SMALL>
 struct EmuCfg {
-  static constexpr int NP2 = NP * NP, NP3 = NP2 * NP, EB = STAGE ? emu_eb_staged(NP) : emu_eb(NP), NT = NP2 * EB;
+  static constexpr int NP2 = NP * NP, NP3 = NP2 * NP, EB = emu_eb(NP, STAGE || SMALL), NT = NP2 * EB;
   static constexpr int RS = NP | 1, PS = NP * RS, BUF = NP * PS;
   static constexpr int GS = (12 * NP3 + 3) / 4 * 4;  // factor block of one element (floats)
   // byte offsets: [factor block (TMA, offset 0)] [value buffers] [reduction slots, mbarrier]
@@ -336,7 +336,8 @@ __host__ __device__ constexpr bool emu_stage_fits(int NP) {
 
 // Blocks per SM the register allocation is held to; 0 = no floor (an explicit 1 lets the compiler
 // take far more registers).  Measured for the packed forms over floors of 0..7.
-__host__ __device__ constexpr int emu_min_blocks(int NP, bool stage, bool dot) {
+__host__ __device__ constexpr int emu_min_blocks(int NP, bool stage, bool dot, bool small) {
+  if (small) return 0;
   if (stage) return NP == 10 ? 4 : NP == 11 ? 3 : NP >= 12 ? 2 : 0;
   if (dot) return NP == 4 ? 7 : NP == 10 || NP >= 12 ? 2 : 0;
   return NP == 4 ? 7 : NP == 6 || NP == 7 ? 4 : NP == 8 ? 5 : NP == 9 || NP == 11 ? 3 : NP >= 10 ? 2 : 0;
@@ -358,9 +359,9 @@ __host__ __device__ constexpr int emu_loop_mode(int NP) {
 // below)
 __host__ __device__ constexpr bool emu_prefetch(int NP) { return NP >= 14; }
 
-template <int NP, bool BOXM, bool STAGE, bool DOT>
-__global__ void __launch_bounds__(EmuCfg<NP, STAGE, DOT>::NT, emu_min_blocks(NP, STAGE, DOT)) k_apply_emu(const EmuParams<NP> P) {
-  using C = EmuCfg<NP, STAGE, DOT>;
+template <int NP, bool BOXM, bool STAGE, bool DOT, bool SMALL>
+__global__ void __launch_bounds__(EmuCfg<NP, STAGE, DOT, SMALL>::NT, emu_min_blocks(NP, STAGE, DOT, SMALL)) k_apply_emu(const EmuParams<NP> P) {
+  using C = EmuCfg<NP, STAGE, DOT, SMALL>;
   constexpr int N = NP - 1, NP2 = C::NP2, NP3 = C::NP3, EB = C::EB, NT = C::NT, RS = C::RS, PS = C::PS,
                 BUF = C::BUF, GS = C::GS;
   constexpr bool PK = emu_packed(NP, DOT);
@@ -713,24 +714,30 @@ __global__ void __launch_bounds__(EmuCfg<NP, STAGE, DOT>::NT, emu_min_blocks(NP,
   }
 }
 
-template <int NP, bool BOXM, bool STAGE, bool DOT>
+template <int NP, bool BOXM, bool STAGE, bool DOT, bool SMALL>
 sem_status launch_k(const EmuParams<NP> &p, cudaStream_t s) {
-  using C = EmuCfg<NP, STAGE, DOT>;
+  using C = EmuCfg<NP, STAGE, DOT, SMALL>;
   const unsigned grid = (unsigned)((p.E + C::EB - 1) / C::EB);
   if (p.partials && grid > SEM_MAX_PARTIALS) return sem_fail(SEM_ERR_INVALID, "too many elements for fused dot");
   static std::atomic<unsigned long long> attr_done;
-  const cudaError_t e = set_smem_limit_once(k_apply_emu<NP, BOXM, STAGE, DOT>, C::SMEM, attr_done);
+  const cudaError_t e = set_smem_limit_once(k_apply_emu<NP, BOXM, STAGE, DOT, SMALL>, C::SMEM, attr_done);
   if (e != cudaSuccess) return sem_fail(SEM_ERR_CUDA, std::string("emu attributes: ") + cudaGetErrorString(e));
-  k_apply_emu<NP, BOXM, STAGE, DOT><<<grid, C::NT, C::SMEM, s>>>(p);
+  k_apply_emu<NP, BOXM, STAGE, DOT, SMALL><<<grid, C::NT, C::SMEM, s>>>(p);
   return SEM_OK;
 }
 
-template <int NP, bool STAGE>
+template <int NP, bool STAGE, bool SMALL>
 sem_status launch_b(const EmuParams<NP> &p, bool boxm, bool dot, cudaStream_t s) {
-  if (dot)
-    return boxm ? launch_k<NP, true, STAGE, true>(p, s) : launch_k<NP, false, STAGE, true>(p, s);
-  return boxm ? launch_k<NP, true, STAGE, false>(p, s) : launch_k<NP, false, STAGE, false>(p, s);
+  if (dot) return boxm ? launch_k<NP, true, STAGE, true, SMALL>(p, s) : launch_k<NP, false, STAGE, true, SMALL>(p, s);
+  return boxm ? launch_k<NP, true, STAGE, false, SMALL>(p, s) : launch_k<NP, false, STAGE, false, SMALL>(p, s);
 }
+
+// Whether a problem is too small for the fuller blocks of emu_eb: these (and their register floors, which
+// spill) serve a chip full of blocks; below two blocks per SM a thread's own latency counts.
+// 27 elements at N = 9 / 11, us: fuller blocks 21.4 / 29.9, smaller 10.6 / 16.0 (with one element per
+// block and the floors: 13.4 / 19.4).
+__host__ __device__ constexpr bool emu_has_small(int NP) { return emu_eb(NP, false) != emu_eb(NP, true); }
+inline bool emu_small(int NP, int64_t E) { return emu_has_small(NP) && E < (int64_t)2 * 152 * emu_eb(NP, false); }
 
 template <int NP>
 sem_status launch_emu(const sem_handle *h, const double *u, double *y, double *partials, SemScalars *scal,
@@ -777,11 +784,13 @@ sem_status launch_emu(const sem_handle *h, const double *u, double *y, double *p
       }
   if (partials && !scal) return sem_fail(SEM_ERR_INVALID, "fused dot needs the solver scalars");
   const bool boxm = p.glo == nullptr && p.bc != SEM_BC_MASK;
-  // variant 0: factor block staged by TMA when it fits; other variants, and automatic (-1), read
-  // factors directly
-  const bool stage = emu_stage_fits(NP) && h->apply_variant == 0;
-  const sem_status st = stage ? launch_b<NP, emu_stage_fits(NP)>(p, boxm, partials != nullptr, s)
-                              : launch_b<NP, false>(p, boxm, partials != nullptr, s);
+  // variant 0: factor block staged by TMA when it fits; other variants read factors directly, and so
+  // does the automatic choice (-1) except on small problems at N = 5 (64 elements: 7.1 against 8.8 us)
+  const bool small = emu_small(NP, p.E);
+  const bool stage = emu_stage_fits(NP) && (h->apply_variant == 0 || (h->apply_variant < 0 && NP == 6 && small));
+  const sem_status st = stage ? launch_b<NP, emu_stage_fits(NP), false>(p, boxm, partials != nullptr, s)
+                        : small ? launch_b<NP, false, emu_has_small(NP)>(p, boxm, partials != nullptr, s)
+                                             : launch_b<NP, false, false>(p, boxm, partials != nullptr, s);
   if (st != SEM_OK) return st;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return sem_fail(SEM_ERR_CUDA, std::string("emu apply launch: ") + cudaGetErrorString(e));
