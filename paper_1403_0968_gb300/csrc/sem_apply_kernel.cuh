@@ -337,8 +337,6 @@ __global__ void __launch_bounds__(ApplyCfg<NP, EB_>::NT, apply_min_blocks<T>(NP,
   double *s_red = reinterpret_cast<double *>(smem_raw + RED_OFF);
   uint64_t *bar = reinterpret_cast<uint64_t *>(smem_raw + RED_OFF + apply_red_size<NP, T, EB_>());
 
-  // inside a solve: nothing to do once the iteration has stopped (flag set by an earlier launch)
-  if (P.scal && (P.scal->converged || P.scal->breakdown)) return;
   const int tid = threadIdx.x;
   const int es = tid / NP2, t2 = tid - es * NP2, a = t2 % NP, b = t2 / NP;
   const int64_t e0 = (int64_t)blockIdx.x * EB;
@@ -346,13 +344,23 @@ __global__ void __launch_bounds__(ApplyCfg<NP, EB_>::NT, apply_min_blocks<T>(NP,
   const bool active = e < P.E;
   T *su = sbuf + es * 3 * BUF, *sr = su + BUF, *ss = sr + BUF;
 
-
   if constexpr (STAGE) {
     if (tid == 0) mbar_init(bar, 1);
     __syncthreads();
     if (tid == 0) {
       const int64_t nel = (P.E - e0) < EB ? (P.E - e0) : EB;
       tma_load_1d(sG, static_cast<const TG *>(P.Gf) + e0 * P.gs, (uint32_t)(nel * P.gs * sizeof(TG)), bar);
+    }
+  }
+  // inside a solve: the kernel before this one has to be complete (the factors, asked for above, depend
+  // on no kernel of the solve); nothing to do once the iteration has stopped
+  if (P.scal) {
+    dependent_wait();
+    if (P.scal->converged || P.scal->breakdown) {
+      if constexpr (STAGE) {
+        if (tid == 0) mbar_wait(bar, 0);  // not before this block's own copy has landed
+      }
+      return;
     }
   }
 
@@ -701,11 +709,17 @@ static sem_status launch_apply_v(const ApplyParams<T, NP> &p, cudaStream_t s) {
                                : set_smem_limit_once(k_apply<NP, T, EB, STAGE, false, TG>, smem, attr_done[0]);
     if (e != cudaSuccess) return sem_fail(SEM_ERR_CUDA, std::string("apply smem attribute: ") + cudaGetErrorString(e));
   }
-  if (boxm)
-    k_apply<NP, T, EB, STAGE, true, TG><<<grid, C::NT, smem, s>>>(p);
-  else
-    k_apply<NP, T, EB, STAGE, false, TG><<<grid, C::NT, smem, s>>>(p);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e;
+  if (p.scal) {  // a step of a solve
+    e = boxm ? launch_dependent(k_apply<NP, T, EB, STAGE, true, TG>, grid, C::NT, smem, s, p)
+             : launch_dependent(k_apply<NP, T, EB, STAGE, false, TG>, grid, C::NT, smem, s, p);
+  } else {
+    if (boxm)
+      k_apply<NP, T, EB, STAGE, true, TG><<<grid, C::NT, smem, s>>>(p);
+    else
+      k_apply<NP, T, EB, STAGE, false, TG><<<grid, C::NT, smem, s>>>(p);
+    e = cudaGetLastError();
+  }
   if (e != cudaSuccess) return sem_fail(SEM_ERR_CUDA, std::string("apply launch: ") + cudaGetErrorString(e));
   return SEM_OK;
 }

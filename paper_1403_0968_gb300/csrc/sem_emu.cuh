@@ -373,7 +373,10 @@ __global__ void __launch_bounds__(EmuCfg<NP, STAGE, DOT, SMALL>::NT, emu_min_blo
   uint64_t *bar = reinterpret_cast<uint64_t *>(smem_raw + C::RED_OFF + C::RED_SIZE);
   int *s_emax = reinterpret_cast<int *>(bar + 2);  // [EB] largest biased FP64 exponent of each element's u
 
-  if (DOT && (P.scal->converged || P.scal->breakdown)) return;
+  if constexpr (DOT) {  // a step of a solve: nothing to do once the iteration has stopped
+    dependent_wait();
+    if (P.scal->converged || P.scal->breakdown) return;
+  }
   const int tid = threadIdx.x;
   const int es = tid / NP2, t2 = tid - es * NP2, a = t2 % NP, b = t2 / NP;
   if (t2 == 0) s_emax[es] = 1;
@@ -722,7 +725,10 @@ sem_status launch_k(const EmuParams<NP> &p, cudaStream_t s) {
   static std::atomic<unsigned long long> attr_done;
   const cudaError_t e = set_smem_limit_once(k_apply_emu<NP, BOXM, STAGE, DOT, SMALL>, C::SMEM, attr_done);
   if (e != cudaSuccess) return sem_fail(SEM_ERR_CUDA, std::string("emu attributes: ") + cudaGetErrorString(e));
-  k_apply_emu<NP, BOXM, STAGE, DOT, SMALL><<<grid, C::NT, C::SMEM, s>>>(p);
+  if constexpr (DOT)
+    SEM_CUDA_TRY(launch_dependent(k_apply_emu<NP, BOXM, STAGE, DOT, SMALL>, grid, C::NT, C::SMEM, s, p));
+  else
+    k_apply_emu<NP, BOXM, STAGE, DOT, SMALL><<<grid, C::NT, C::SMEM, s>>>(p);
   return SEM_OK;
 }
 

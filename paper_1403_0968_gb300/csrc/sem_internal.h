@@ -149,6 +149,31 @@ cudaError_t set_smem_limit_once(K *kernel, size_t bytes, std::atomic<unsigned lo
   return e;
 }
 
+// ----- programmatic dependent launch -----
+// The kernels of a CG iteration depend on one another in a chain.  Launched with launch_dependent, a
+// kernel is set up while the one before it drains; dependent_wait at its start returns when that kernel
+// has completed and its writes are visible (at once in a plain launch).  Every kernel launched this way
+// calls dependent_wait before it reads or writes anything that a kernel before it touches, so the chain
+// stays as ordered as plain launches are.  6^3 / 16^3 elements, N = 7, per iteration: 20.9 -> 19.7 / 37.8 ->
+// 37.3 us (with the dependents let in before the end, griddepcontrol.launch_dependents: 20.3 / 38.9).
+__device__ __forceinline__ void dependent_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
+                             A &&...args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // GLL points x, weights w (N + 1 each) and derivative matrix D[i][j] = l_j'(x_i) (row-major) of
 // order N, in FP64 on the host
 void sem_gll_tables(int N, double *x, double *w, double *D);

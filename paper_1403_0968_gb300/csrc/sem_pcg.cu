@@ -98,6 +98,7 @@ __global__ void __launch_bounds__(UT, 2) k_cg_update(int64_t G, T *__restrict__ 
   __shared__ T s_part[2][UT];
   __shared__ double s_tot[2];
   __shared__ int s_last;
+  dependent_wait();
   if (S->converged || S->breakdown) return;
   const T alpha = (T)S->alpha;
   const int tid = threadIdx.x, warp = tid >> 5;
@@ -164,6 +165,7 @@ template <typename T>
 __global__ void __launch_bounds__(UT, 2) k_cg_direction(int64_t G, T *__restrict__ p, const T *__restrict__ r,
                                                         T *__restrict__ Ap, const T *__restrict__ dinv,
                                                         const SemScalars *S) {
+  dependent_wait();
   if (S->converged || S->breakdown) return;
   const T beta = (T)S->beta;
   using V = Vec16<T>;
@@ -417,10 +419,11 @@ sem_status cg_block(sem_handle *h, int prec, int count, T *x, T *p, T *r, T *Ap,
     if (s != SEM_OK) return s;
     const unsigned grid = ugrid(h->G, Vec16<T>::N);
     if (reinterpret_cast<uintptr_t>(x) % 16 == 0)
-      k_cg_update<T, true><<<grid, UT, 0, st>>>(h->G, x, p, r, Ap, dinv, h->scal, h->partials);
+      SEM_CUDA_TRY(launch_dependent(k_cg_update<T, true>, grid, UT, 0, st, h->G, x, p, r, Ap, dinv, h->scal, h->partials));
     else
-      k_cg_update<T, false><<<ugrid(h->G, 1), UT, 0, st>>>(h->G, x, p, r, Ap, dinv, h->scal, h->partials);
-    k_cg_direction<T><<<grid, UT, 0, st>>>(h->G, p, r, Ap, dinv, h->scal);
+      SEM_CUDA_TRY(launch_dependent(k_cg_update<T, false>, ugrid(h->G, 1), UT, 0, st, h->G, x, p, r, Ap, dinv, h->scal,
+                                    h->partials));
+    SEM_CUDA_TRY(launch_dependent(k_cg_direction<T>, grid, UT, 0, st, h->G, p, r, Ap, dinv, h->scal));
   }
   SEM_CUDA_TRY(cudaGetLastError());
   return SEM_OK;
