@@ -214,37 +214,37 @@ __global__ void k_mlp_scatter(sem_handle h, const float *O, const float *scale, 
 
 // structured box: z[g] = (1 / multiplicity) sum over the elements containing g of scale_e O[e][p]
 // (FP32, fixed order: no atomics, deterministic) plus D^-1 r with the Jacobi base; zero on
-// Dirichlet nodes.  One thread per global node (I, J, K) on a 3-D grid (x by blocks of threads, y
-// and z by grid rows).  Along each direction a lattice index lies inside one element or, on an
-// inner element face, in two: the lower element's local index N and the upper one's 0; the
-// multiplicity is 2 per such direction.  J and K are the same for the whole block, so the (y, z)
-// element pairs and their row offsets are worked out once per block; each thread adds its one or
-// two x-neighbours per pair (order: z lower to upper, then y, then x, as the sum is defined).
+// Dirichlet nodes.  A block takes GTH consecutive nodes of one z plane (K by grid row), so that every
+// thread of every block but a plane's last has a node (rows of 225 nodes left an eighth of 2 x 128
+// threads idle).  Along each direction a lattice index lies inside one element or, on an inner element
+// face, in two: the lower element's local index N and the upper one's 0; the multiplicity is 2 per such
+// direction (order of the sum: z lower to upper, then y, then x).  340 MB at 32^3 elements, N = 7 (51 us at the copy rate), about 75 us:
+// most of it instruction issue (some 150 per node).  Whole preconditioner there 166.3 -> 163.0 us with
+// this split; two or four nodes per thread 164.2 / 164.3, 256 threads 166.3.
+constexpr int GTH = 128;
 template <int NP>
-__global__ void __launch_bounds__(128) k_mlp_gather(sem_handle h, const float *__restrict__ O,
+__global__ void __launch_bounds__(GTH) k_mlp_gather(sem_handle h, const float *__restrict__ O,
                                                     const float *__restrict__ scale, const double *__restrict__ r,
                                                     double *__restrict__ z) {
   constexpr int N = NP - 1, N3 = NP * NP * NP;
   const int sx = h.box[0], sy = h.box[1], sz = h.box[2];
-  const int gxs = sx * N + 1, gys = sy * N + 1;
-  const int I = blockIdx.x * blockDim.x + threadIdx.x, J = blockIdx.y, K = blockIdx.z;
-  // block-uniform: the (element row, local row) pairs in y and z
-  const int eya = J / N < sy ? J / N : sy - 1, ja = J - eya * N;
+  const int gxs = sx * N + 1, gys = sy * N + 1, K = blockIdx.y;
+  const int64_t plane = (int64_t)gxs * gys, g0 = plane * K;
+  const uint32_t q = blockIdx.x * GTH + threadIdx.x;  // node of the plane
+  if (q >= plane) return;
   const int eza = K / N < sz ? K / N : sz - 1, ka = K - eza * N;
-  const bool y2 = ja == 0 && eya > 0, z2 = ka == 0 && eza > 0;
-  if (I >= gxs) return;
-  const int64_t g = I + (int64_t)gxs * (J + (int64_t)gys * K);
-  // both node values are loaded up front, independent of each other and of the element outputs
-  // (r is read on Dirichlet nodes too, where it is not used), so that the loads overlap
+  const bool z2 = ka == 0 && eza > 0;
+  // node values up front, independent of each other and of the element outputs (r is read on Dirichlet
+  // nodes too, where it is not used), so that the loads overlap
+  const int64_t g = g0 + q;
   const double dv = __ldg(h.dinv64 + g), rv = __ldg(r + g);
+  const int J = q / (uint32_t)gxs, I = q - J * gxs;
+  const int eya = J / N < sy ? J / N : sy - 1, ja = J - eya * N;
   const int exa = I / N < sx ? I / N : sx - 1, ia = I - exa * N;
-  const bool x2 = ia == 0 && exa > 0;
+  const bool y2 = ja == 0 && eya > 0, x2 = ia == 0 && exa > 0;
   float acc = 0.f;
-  // block-uniform trip counts (1 or 2 each): the loops run over the pairs that exist only
-#pragma unroll 1
   for (int zc = z2 ? 0 : 1; zc < 2; ++zc) {
     const int ez = zc == 0 ? eza - 1 : eza, iz = zc == 0 ? N : ka;
-#pragma unroll 1
     for (int yc = y2 ? 0 : 1; yc < 2; ++yc) {
       const int ey = yc == 0 ? eya - 1 : eya, iy = yc == 0 ? N : ja;
       const int64_t erow = (int64_t)sx * (ey + (int64_t)sy * ez);  // first element of this x row
@@ -359,11 +359,13 @@ sem_status sem_mlp_precond_apply(sem_handle *h, const double *r, double *z, cuda
   } else {
     const int64_t gx3 = (int64_t)h->box[0] * h->N + 1, gy3 = (int64_t)h->box[1] * h->N + 1,
                   gz3 = (int64_t)h->box[2] * h->N + 1;
-    if (gy3 > 65535 || gz3 > 65535) return sem_fail(SEM_ERR_INVALID, "box too large for the gather grid");
+    // (a plane's nodes have 32-bit indices: more would not fit the device)
+    if (gy3 > 65535 || gz3 > 65535 || gx3 * gy3 > 0xfffff000ll)
+      return sem_fail(SEM_ERR_INVALID, "box too large for the gather grid");
     switch (h->n) {
 #define SEM_GT(NPV)                                                                                   \
   case NPV:                                                                                         \
-    k_mlp_gather<NPV><<<dim3((unsigned)((gx3 + 127) / 128), (unsigned)gy3, (unsigned)gz3), 128, 0, st>>>( \
+    k_mlp_gather<NPV><<<dim3((unsigned)((gx3 * gy3 + GTH - 1) / GTH), (unsigned)gz3), GTH, 0, st>>>( \
         *h, h->mlp_O, h->mlp_scale, r, z);                                                          \
     break;
       SEM_GT(2) SEM_GT(3) SEM_GT(4) SEM_GT(5) SEM_GT(6) SEM_GT(7) SEM_GT(8) SEM_GT(9) SEM_GT(10) SEM_GT(11)
