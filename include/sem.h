@@ -177,13 +177,14 @@ sem_status sem_set_wait_limit(sem_handle *h, int64_t polls);
  * and whether the per-element factor block is staged in shared memory by a bulk TMA copy):
  *   -1 automatic (the default after sem_setup): a per-order choice measured on GB300;
  *   0 default elements per block, factors staged (when they fit); 1 default, factors read from
- *   global memory; 2 twice the elements per block, factors from global; 3 half the elements per
- *   block, staged; 4 persistent blocks that double-buffer the next tile's factors by TMA and
- *   prefetch its u (structured boxes; otherwise as 0); 5 (order 7 only: the D-contractions on
- *   the tensor cores — SEM_FP64_EMU by exact TF32 slicing to its FP64 accuracy, SEM_FP32 by
- *   two-slice TF32 ("3xTF32") with FP32 accumulation, about 2^-22 of |D||v| per line product;
- *   at other orders SEM_FP64_EMU treats 5 as 1 and the other precisions as 0; on GB300 both
- *   measured slower than their CUDA-core kernels, which stay the automatic choice).
+ *   global memory (SEM_FP64 where it is the faster form, most orders and sizes from 3 to 14: one
+ *   element per block, three threads per column); 2 twice the elements per block, factors from
+ *   global; 3 half the elements per block, staged; 4 persistent blocks that double-buffer the next
+ *   tile's factors by TMA and prefetch its u (structured boxes; otherwise as 0); 5 (order 7 only:
+ *   the D-contractions on the tensor cores — SEM_FP64_EMU by exact TF32 slicing to its FP64
+ *   accuracy, SEM_FP32 by two-slice TF32 ("3xTF32") with FP32 accumulation, about 2^-22 of |D||v|
+ *   per line product; at other orders SEM_FP64_EMU treats 5 as 1 and the other precisions as 0; on
+ *   GB300 both measured slower than their CUDA-core kernels, which stay the automatic choice).
  *   SEM_FP64_EMU distinguishes 0 (staged) from 1..4 (direct reads); SEM_FP32_OTF has no factor
  *   block, so 0, 1 and 4 coincide.
  * All variants compute the same operator (results differ by the order of the atomic scatter-add

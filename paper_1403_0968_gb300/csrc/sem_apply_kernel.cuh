@@ -731,7 +731,8 @@ __host__ __device__ constexpr size_t pipe_smem();
 
 // Kernel variants an order can run (the autotuner picks one per problem):
 //   0  default elements per block, factor block staged by TMA (when it fits)
-//   1  default elements per block, factors read straight from global memory
+//   1  default elements per block, factors read straight from global memory (FP64: k_apply_cols where
+//      apply_cols says so)
 //   2  twice the elements per block, factors from global memory
 //   3  half the elements per block (at least 1), factors staged by TMA (when it fits)
 //   4  persistent blocks, next tile's factors double-buffered by TMA and its u prefetched
@@ -742,8 +743,8 @@ __host__ __device__ constexpr size_t pipe_smem();
 // nodes, variants 0 / 1 / 3): FP32 N = 2 116 / 109 / 113, 3 108 / 121 / 111, 5 107 / 111 / 110, 6 110 / 93 /
 // 113, 7 122 / 100 / 116, 15 56 / 56 / 56 (the former choice there, 2: 49); BF16 N = 2 141 / 120 / 136, 3
 // 145 / 127 / 145, 5 130 / 108 / 114, 6 135 / 105 / 140, 7 144 / 106 / 139, 15 74 / 58 / 74; on the fly
-// (no factor block: 0 = 1) N = 3 139 / 139, 5 126 / 97, 6 120 / 116, 7 147 / 155 (variants 1 / 3).  FP64 is
-// bound by its FMA pipe and indifferent.
+// (no factor block: 0 = 1) N = 3 139 / 139, 5 126 / 97, 6 120 / 116, 7 147 / 155 (variants 1 / 3).  FP64
+// takes 1 (k_apply_cols where it is the faster one).
 template <typename T, typename TG>
 __host__ __device__ constexpr int apply_auto_variant(int NP) {
   return is_otf<TG>() ? (NP == 4 || NP == 8 ? 3 : 1)
@@ -753,9 +754,180 @@ __host__ __device__ constexpr int apply_auto_variant(int NP) {
          : (NP == 3 || (NP > 6 && NP < 16)) ? 0 : 1;
 }
 
+// FP64 apply with one element per block and three threads for every column of it instead of one: the line
+// products of the three directions run side by side (group d of the threads takes direction d in phases 1
+// and 3), and the nodes of a column are dealt to the groups in the other phases.
+//
+// Bound: GB300 issues a warp's FP64 instruction over about 16 cycles of the SM, so the FMA pipe sets the
+// time of a large problem if enough warps are there to fill it, and one element's chain of instructions
+// sets that of a small one.  A thread of k_apply holds a line, its column's intermediates and factors at
+// once (N = 11: one block of 144 threads per SM and scheduler gaps); here it holds one line, and three
+// times the warps share an element.  k_apply / this kernel: us at N = 7 with 64 elements 19.2 / 12.5; GDOF/s
+// at 8e6 nodes N = 3 13.2 / 10.3, 4 12.3 / 11.1, 5 10.4 / 10.4, 6 9.2 / 10.9, 7 10.6 / 10.7, 8 8.7 / 9.7, 9 7.5 /
+// 8.8, 10 8.2 / 8.6, 11 5.8 / 8.1, 12 6.2 / 7.9, 13 6.0 / 7.1, 14 6.0 / 6.9, 15 6.4 / 6.2.  FP32 and BF16
+// factors have warps enough in k_apply and lose to the extra passes through shared memory (N = 7: 123 / 60
+// and 144 / 50), so the form is FP64's alone.
+//
+// Registers: small orders ask for their factors with u, beside the gather and the gradients (an element
+// alone on an SM waits for them otherwise); from N = 9 those registers are worth more as resident blocks
+// (N = 9 at 8e6 nodes: 6.8 with the factors held, 8.2 without, 8.8 at three blocks per SM).
+constexpr int cols_min_blocks(int NP) { return NP <= 9 ? 1 : NP == 10 ? 3 : 2; }
+
+// Orders and sizes it is for (k_apply / this kernel): N = 5 to 9, 11 and 12 at every size (N = 5: 64 elements
+// 13.7 / 7.6 us, 2744 69.0 / 64.2; N = 7: 216 elements 19.3 / 19.6, faster elsewhere; N = 12: 27 elements 48.6 /
+// 48.4); N = 3 and 4, whose k_apply blocks hold 8 and 5 elements, up to four and three elements per SM (N = 3:
+// 729 elements 9.9 / 9.1, 1000 10.0 / 10.8; N = 4: 343 11.7 / 9.4, 512 11.7 / 11.1, 729 11.7 / 13.0); N = 13 and 14
+// from two elements per SM (N = 13: 125 elements 62.7 / 64.7, 8e6 nodes 6.0 / 7.1 GDOF/s).  Not N = 10 (125
+// elements 28.3 / 30.1, 343 74 / 81), and not N = 15, which spills at the 80 registers that are left.
+constexpr bool apply_cols(int NP, int64_t E) {
+  return NP == 4 ? E <= 4 * 152 : NP == 5 ? E <= 3 * 152 : NP == 14 || NP == 15 ? E > 2 * 152 : NP >= 6 && NP <= 13 && NP != 11;
+}
+
+template <int NP, bool BOXM>
+__global__ void __launch_bounds__(3 * NP * NP, cols_min_blocks(NP)) k_apply_cols(const ApplyParams<double, NP> P) {
+  using T = double;
+  constexpr int N = NP - 1, NP2 = NP * NP, NP3 = NP2 * NP, NT = 3 * NP2, RS = NP | 1, PS = NP * RS, BUF = NP * PS;
+  constexpr int MK = (NP + 2) / 3;  // nodes of a column per group: k = grp, grp + 3, ...
+  constexpr bool PF = NP <= 9;      // the factors asked for with u, beside the gather and the gradients
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  T *su = reinterpret_cast<T *>(smem_raw), *sv = su + BUF;  // u, then r, s and t lines
+  if (P.scal) {
+    dependent_wait();
+    if (P.scal->converged || P.scal->breakdown) return;
+  }
+  const int tid = threadIdx.x, grp = tid / NP2, t2 = tid - grp * NP2, a = t2 % NP, b = t2 / NP;
+  const int64_t e = blockIdx.x, plane = P.gxs * P.gys;
+  int64_t gbase = 0;
+  if (BOXM || !P.glo) {  // a general mesh has no box sizes
+    const int64_t ex = e % P.sx, exy = e / P.sx, ey = exy % P.sy, ez = exy / P.sy;
+    gbase = (ex * N + a) + P.gxs * ((ey * N + b) + P.gys * (ez * N));
+  }
+  const T *Ge = static_cast<const T *>(P.Gf) + e * P.gs + t2;
+  int64_t gid[MK];
+  bool dir[MK];
+  T u[MK], gf[MK][6];
+#pragma unroll
+  for (int m = 0; m < MK; ++m) {
+    const int k = grp + 3 * m;
+    if (k >= NP) continue;
+    if constexpr (PF) {
+#pragma unroll
+      for (int f = 0; f < 6; ++f) gf[m][f] = Ge[f * NP3 + k * NP2];
+    }
+    const int64_t g = BOXM || !P.glo ? gbase + k * plane : (int64_t)P.glo[e * NP3 + t2 + NP2 * k];
+    bool d = false;
+    if (P.bc == SEM_BC_BOX) {
+      const int64_t I = g % P.gxs, J = (g / P.gxs) % P.gys, K = g / plane;
+      d = I == 0 || J == 0 || K == 0 || I == P.gxs - 1 || J == P.gys - 1 || K == P.gzs - 1;
+    } else if (!BOXM && P.bc == SEM_BC_MASK) {
+      d = P.mask[g] != 0;
+    }
+    gid[m] = g;
+    dir[m] = d;
+    u[m] = d ? T(0) : P.u[g];
+    su[k * PS + b * RS + a] = u[m];
+  }
+  __syncthreads();
+  // the group's line: r (j = a, k = b), s (i = a, k = b) or t (i = a, j = b)
+  const int lb = grp == 0 ? b * PS + a * RS : grp == 1 ? b * PS + a : b * RS + a;
+  const int ls = grp == 0 ? 1 : grp == 1 ? RS : PS;
+  T *sg = sv + grp * BUF;
+  {
+    T row[NP], out[NP];
+#pragma unroll
+    for (int m = 0; m < NP; ++m) row[m] = su[lb + m * ls];
+    line_apply<NP, T, false>(P.D, 0, row, out);
+#pragma unroll
+    for (int m = 0; m < NP; ++m) sg[lb + m * ls] = out[m];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int m = 0; m < MK; ++m) {
+    const int k = grp + 3 * m, q = k * PS + b * RS + a;
+    if (k >= NP) continue;
+    if constexpr (!PF) {
+#pragma unroll
+      for (int f = 0; f < 6; ++f) gf[m][f] = Ge[f * NP3 + k * NP2];
+    }
+    const T ur = sv[q], us = sv[BUF + q], ut = sv[2 * BUF + q];
+    sv[q] = gf[m][0] * ur + gf[m][1] * us + gf[m][2] * ut;
+    sv[BUF + q] = gf[m][1] * ur + gf[m][3] * us + gf[m][4] * ut;
+    sv[2 * BUF + q] = gf[m][2] * ur + gf[m][4] * us + gf[m][5] * ut;
+  }
+  __syncthreads();
+  {
+    T row[NP], out[NP];
+#pragma unroll
+    for (int m = 0; m < NP; ++m) row[m] = sg[lb + m * ls];
+    line_apply<NP, T, false>(P.D, 1, row, out);
+#pragma unroll
+    for (int m = 0; m < NP; ++m) sg[lb + m * ls] = out[m];  // a line is read and written by its own thread only
+  }
+  __syncthreads();
+  T dotp = T(0), y[MK];
+#pragma unroll
+  for (int m = 0; m < MK; ++m) {
+    const int k = grp + 3 * m, q = k * PS + b * RS + a;
+    if (k >= NP) continue;
+    y[m] = sv[2 * BUF + q] + sv[q] + sv[BUF + q];
+    if (P.wJa) y[m] += P.wJa[e * NP3 + t2 + NP2 * k] * u[m];
+    if (!dir[m]) dotp += u[m] * y[m];
+  }
+  if (P.partials) {
+    su[tid] = dotp;  // u has been read for the last time; NT <= BUF
+    __syncthreads();
+    if (tid < 32) {
+      double pAp;
+      if (warp_publish_2level(warp_sum(su, NT), P.partials, P.gpartials, P.gtickets, &P.scal->counter[0], &pAp) &&
+          tid == 0)
+        cg_set_alpha(P.scal, pAp);
+    }
+  }
+  const bool ij_interior = a > 0 && a < N && b > 0 && b < N && (BOXM || !P.glo);
+#pragma unroll
+  for (int m = 0; m < MK; ++m) {
+    const int k = grp + 3 * m;
+    if (k >= NP || dir[m]) continue;
+    if (ij_interior && k > 0 && k < N)
+      P.y[gid[m]] = y[m];  // no other element touches the node
+    else
+      atomicAdd(P.y + gid[m], y[m]);
+  }
+}
+
+template <int NP>
+static sem_status launch_apply_cols(const ApplyParams<double, NP> &p, cudaStream_t s) {
+  constexpr int NT = 3 * NP * NP;
+  static_assert(NP >= 4 && NT <= 1024, "a full warp for the fused sum; 3 NP^2 <= NP^2 (NP | 1)");
+  constexpr size_t smem = (size_t)(4 * NP * NP * (NP | 1)) * sizeof(double);
+  const bool boxm = p.glo == nullptr && p.bc != SEM_BC_MASK;
+  static std::atomic<unsigned long long> attr_done[2];
+  cudaError_t e = boxm ? set_smem_limit_once(k_apply_cols<NP, true>, smem, attr_done[1])
+                       : set_smem_limit_once(k_apply_cols<NP, false>, smem, attr_done[0]);
+  if (e == cudaSuccess) {
+    if (p.scal) {  // a step of a solve
+      e = boxm ? launch_dependent(k_apply_cols<NP, true>, (unsigned)p.E, NT, smem, s, p)
+               : launch_dependent(k_apply_cols<NP, false>, (unsigned)p.E, NT, smem, s, p);
+    } else {
+      if (boxm)
+        k_apply_cols<NP, true><<<(unsigned)p.E, NT, smem, s>>>(p);
+      else
+        k_apply_cols<NP, false><<<(unsigned)p.E, NT, smem, s>>>(p);
+      e = cudaGetLastError();
+    }
+  }
+  if (e != cudaSuccess) return sem_fail(SEM_ERR_CUDA, std::string("apply launch: ") + cudaGetErrorString(e));
+  return SEM_OK;
+}
+
 template <int NP, typename T, typename TG = T>
 static sem_status launch_apply_np(const ApplyParams<T, NP> &p, int variant, cudaStream_t s) {
   if (variant < 0) variant = apply_auto_variant<T, TG>(NP);
+  if constexpr (std::is_same<T, double>::value && NP >= 4 && NP <= 15 && NP != 11) {
+    // (a solve's fused sum takes one partial per block; beyond that many elements, k_apply's larger blocks)
+    if (variant == 1 && p.batch == nullptr && apply_cols(NP, p.E) && (!p.partials || p.E <= SEM_MAX_PARTIALS))
+      return launch_apply_cols<NP>(p, s);
+  }
   constexpr int EB0 = apply_eb_default(NP);
   constexpr int EB2 = (EB0 * 2 * NP * NP <= 1024 &&
                        apply_smem<NP, T, EB0 * 2, false, TG>() <= SEM_MAX_SMEM_PER_BLOCK) ? EB0 * 2 : EB0;
