@@ -241,7 +241,8 @@ struct EmuParams {
 __host__ __device__ constexpr bool emu_packed(int NP, bool dot) {
   return NP == 4 || NP == 10 || NP >= 12 || (!dot && NP >= 6 && NP <= 9);
 }
-// whether the even and odd parts of a line are formed together too (N = 15 without 26, with 22 GDOF/s)
+// whether the even and odd parts of a line are formed together too (N = 15 one after the other: 26 GDOF/s
+// against 22 in the build the form was chosen in, where its 128 registers did not hold both; 21.3 now)
 __host__ __device__ constexpr bool emu_packed_parts(int NP) { return NP <= 14; }
 
 // out = M v for one line, M = D (TRANS false) or D^T (TRANS true), in double-float: the odd part
@@ -349,14 +350,13 @@ __host__ __device__ constexpr int emu_min_blocks(int NP, bool stage, bool dot, b
 // memory).  The loops shorten the code (fewer instruction-fetch stalls) at some addressing cost.
 // Packed forms, GDOF/s at 1.6e7 nodes, modes 0 / 2 / 3: N = 3 61 / 59 / 55, 5 48 / 47 / 45, 6 41 / 43 /
 // 40, 7 41.5 / 44.5 / 40, 8 34.5 / 36.5 / 35, 9 31.6 / 31.0 / 30.8, 11 23.5 / 24.6 / 23.7, 12 23.5 / 19 /
-// 19, 13 16 / 17 / 20, 14 19 / 12 / 24, 15 16 / 13 / 26.
+// 19, 13 16 / 17 / 20; mode 3 also leads at N = 14 and 15 (20.5 and 21.3 as chosen here).
 __host__ __device__ constexpr int emu_loop_mode(int NP) {
   return NP >= 14 ? 3 : (NP == 7 || NP == 8 || NP == 9 || NP == 11 || NP == 12) ? 2 : 0;
 }
 
 // the block's factors asked for in L2 at its start by one bulk prefetch (one element per block and
-// two blocks per SM leave the loads exposed: N = 13 16.9 -> 19.9, 15 24.3 -> 26.2 GDOF/s; slower
-// below)
+// two blocks per SM leave the loads exposed: N = 13 16.9 -> 19.9 GDOF/s, 15 +8%; slower below)
 __host__ __device__ constexpr bool emu_prefetch(int NP) { return NP >= 14; }
 
 template <int NP, bool BOXM, bool STAGE, bool DOT, bool SMALL>
