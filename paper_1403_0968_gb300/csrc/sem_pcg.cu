@@ -72,6 +72,9 @@ __global__ void __launch_bounds__(VT) k_cg_init(int64_t G, const double *b, doub
 
 // The two vector kernels of a CG iteration walk the vectors 16 bytes at a time: UT threads per block,
 // at most two blocks per SM, each thread with the loads of two steps in flight.
+// Vectors that a kernel only reads, but the ones before it write, are not __restrict__: as dependent launches
+// these kernels begin before the writer has ended, and the read-only load path is for data that nothing
+// writes while the kernel lives.
 constexpr int UT = 512, UBLOCKS = 152 * 2;
 
 template <typename T>
@@ -88,9 +91,9 @@ struct alignas(16) Vec16 {
 // FP32: 22 us with 1216 blocks and a butterfly on every warp of each, 13.7 us now (caches
 // flushed before both).
 template <typename T, bool VEC>
-__global__ void __launch_bounds__(UT, 2) k_cg_update(int64_t G, T *__restrict__ x, const T *__restrict__ p,
-                                                     T *__restrict__ r, const T *__restrict__ Ap,
-                                                     const T *__restrict__ dinv, SemScalars *S, double *partials) {
+__global__ void __launch_bounds__(UT, 2) k_cg_update(int64_t G, T *__restrict__ x, const T *p, T *__restrict__ r,
+                                                     const T *Ap, const T *__restrict__ dinv, SemScalars *S,
+                                                     double *partials) {
   constexpr int N = VEC ? Vec16<T>::N : 1;
   struct alignas(N * sizeof(T)) V {
     T v[N];
@@ -162,7 +165,7 @@ __global__ void __launch_bounds__(UT, 2) k_cg_update(int64_t G, T *__restrict__ 
 }
 
 template <typename T>
-__global__ void __launch_bounds__(UT, 2) k_cg_direction(int64_t G, T *__restrict__ p, const T *__restrict__ r,
+__global__ void __launch_bounds__(UT, 2) k_cg_direction(int64_t G, T *__restrict__ p, const T *r,
                                                         T *__restrict__ Ap, const T *__restrict__ dinv,
                                                         const SemScalars *S) {
   dependent_wait();
