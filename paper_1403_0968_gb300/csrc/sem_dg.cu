@@ -183,15 +183,16 @@ __device__ __forceinline__ void dg_fma(float *a, const float *d, float x) {
 }
 __device__ __forceinline__ void dg_fma(double *a, const double *d, double x) { *a = fma(*d, x, *a); }
 
-// 1 / h by one Newton step on the hardware's approximation (within a unit in the last place of the
-// correctly rounded value), without the branch of a full division, which would keep the fluxes of
-// the next node apart from the products of this one; the approximation itself is kept where the
-// step has no meaning (h zero or infinite)
+// 1 / h: one Newton-Raphson step on the hardware's approximation in its fused form, r + r (1 - h r) (Markstein,
+// IBM J. Res. Dev. 34, 1990), within a unit in the last place of the quotient.  A division's branch would
+// keep the fluxes of the next node apart from the products of this one (212,800 triangles, FP32, N = 7: 107
+// against 99 us).  The approximation itself is kept where the step has no meaning: h zero, infinite or so small
+// that its reciprocal overflows (the error is then NaN or infinite).
 __device__ __forceinline__ float dg_reciprocal(float h) {
   float r;
   asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(h));
   const float e = fmaf(-h, r, 1.f);
-  return e == e ? fmaf(r, e, r) : r;
+  return fabsf(e) < 1.f ? fmaf(r, e, r) : r;
 }
 __device__ __forceinline__ double dg_reciprocal(double h) { return 1.0 / h; }
 
