@@ -147,6 +147,13 @@ void vandermonde(int N, std::vector<double> &V, std::vector<double> &Vr, std::ve
 // products; FP32 products run two rows to an instruction (FFMA2: the scalar FMA rate at half the
 // issue slots).  A warp stages the fields of its WE elements by asynchronous copies, one batch ahead,
 // and its results leave through the same buffer; warps are independent of one another.
+//
+// Rounding: the products of SG * RS nodes are summed on their own and then added to the output, so that most
+// roundings happen at a fraction of its size (one addition in 8 to 14 products).  RMS error against FP64,
+// FP32, of each node's pair of products added to the output / one chain of all products / these groups:
+// N = 3 8.76e-8 / 9.12e-8 / 8.22e-8, 5 1.05e-7 / 1.13e-7 / 9.2e-8, 7 1.40e-7 / 1.48e-7 / 1.22e-7, 8 1.72e-7 /
+// 1.82e-7 / 1.58e-7.  At N = 1 and 2 (3 and 6 nodes) groups gain nothing: pairs there.
+//
 // What bounds it at N = 7, FP32: the operator loads (each returns 512 bytes to registers, four
 // cycles of the SM's shared-memory path, for 12 FMA cycles per scheduler) and the FMA pipe, half
 // busy; with the products left out the copies alone take 48 us of the 99 us.  212,800 triangles,
@@ -160,6 +167,9 @@ struct DgCfg {
   static constexpr int RW = sizeof(T) == 4 ? 2 : 1;         // rows per product instruction
   static constexpr int RI = ((NP + RS - 1) / RS + RW - 1) / RW * RW;  // rows per lane
   static constexpr int RP = (RI + VW - 1) / VW * VW;        // row stride of an operator column
+  static constexpr bool PAIR = N <= 2;                      // a node's two products join the sum by themselves
+  // else the products of SG * RS nodes do (a divisor of Np where there is one near)
+  static constexpr int SG = PAIR || RS == 4 ? 1 : RS == 2 ? (N == 6 ? 2 : 3) : N == 5 ? 7 : 5;
   static constexpr int QW = WE * 3 * NP, BW = WE * 2 * NP;  // field and bathymetry values of a batch
   static constexpr int PW = 2 * QW + BW;                    // values staged per warp (fields twice)
   static constexpr int DW = NP * RS * 2 * RP;               // operator values per block
@@ -176,12 +186,22 @@ struct alignas(V * sizeof(T)) DgVec {
   T v[V];
 };
 
-// acc += operator rows times one flux value (two rows to an instruction in FP32)
+// a = operator rows times one flux value, a += the same, a += b (two rows to an instruction in FP32)
+__device__ __forceinline__ void dg_mul(float *a, const float *d, float x) {
+  const float2 r = __fmul2_rn(make_float2(d[0], d[1]), make_float2(x, x));
+  a[0] = r.x, a[1] = r.y;
+}
 __device__ __forceinline__ void dg_fma(float *a, const float *d, float x) {
   const float2 r = __ffma2_rn(make_float2(d[0], d[1]), make_float2(x, x), make_float2(a[0], a[1]));
   a[0] = r.x, a[1] = r.y;
 }
+__device__ __forceinline__ void dg_add(float *a, const float *b) {
+  const float2 r = __fadd2_rn(make_float2(a[0], a[1]), make_float2(b[0], b[1]));
+  a[0] = r.x, a[1] = r.y;
+}
+__device__ __forceinline__ void dg_mul(double *a, const double *d, double x) { *a = *d * x; }
 __device__ __forceinline__ void dg_fma(double *a, const double *d, double x) { *a = fma(*d, x, *a); }
+__device__ __forceinline__ void dg_add(double *a, const double *b) { *a += *b; }
 
 // 1 / h: one Newton-Raphson step on the hardware's approximation in its fused form, r + r (1 - h r) (Markstein,
 // IBM J. Res. Dev. 34, 1990), within a unit in the last place of the quotient.  A division's branch would
@@ -218,7 +238,7 @@ __global__ void __launch_bounds__(32 * DgCfg<T, N, RS_>::W)
     k_dg_volume(int64_t E, T g, const T *__restrict__ ops, const T *__restrict__ Q, const T *__restrict__ Bxy,
                 const T *__restrict__ geo, T *__restrict__ rhs, int wide) {
   using C = DgCfg<T, N, RS_>;
-  constexpr int NP = C::NP, RS = C::RS, WE = C::WE, RI = C::RI, RP = C::RP, VW = C::VW, W = C::W;
+  constexpr int NP = C::NP, RS = C::RS, WE = C::WE, RI = C::RI, RP = C::RP, VW = C::VW, W = C::W, SG = C::SG;
   constexpr int LD = dg_ld(N, sizeof(T));
   extern __shared__ __align__(16) unsigned char dg_smem[];
   T *sD = reinterpret_cast<T *>(dg_smem);
@@ -275,31 +295,50 @@ __global__ void __launch_bounds__(32 * DgCfg<T, N, RS_>::W)
     T x[6], xn[6];
     flux(part, x);
 #pragma unroll 1
-    for (int j0 = 0; j0 < NP; j0 += RS) {
-      flux(j0 + RS + part, xn);
+    for (int j0 = 0; j0 < NP; j0 += SG * RS) {
+      T sum[3][RI];  // this group's products
 #pragma unroll
-      for (int k = 0; k < RS; ++k) {  // node j0 + (part ^ k), from the lane that owns it
-        T y[6];
+      for (int g = 0; g < SG; ++g) {
+        const int js = j0 + g * RS;
+        if (NP % (SG * RS) != 0 && g > 0 && js >= NP) break;
+        flux(js + RS + part, xn);
 #pragma unroll
-        for (int f = 0; f < 6; ++f) y[f] = k == 0 ? x[f] : __shfl_xor_sync(0xffffffffu, x[f], k * WE);
-        const int jk = j0 + (part ^ k), jc = NP % RS == 0 || jk < NP ? jk : NP - 1;
-        const DgVec<T, VW> *d = reinterpret_cast<const DgVec<T, VW> *>(sD + (jc * RS + part) * 2 * RP);
+        for (int k = 0; k < RS; ++k) {  // node js + (part ^ k), from the lane that owns it
+          T y[6];
 #pragma unroll
-        for (int q = 0; q < RP / VW; ++q) {
+          for (int f = 0; f < 6; ++f) y[f] = k == 0 ? x[f] : __shfl_xor_sync(0xffffffffu, x[f], k * WE);
+          const int jk = js + (part ^ k), jc = NP % RS == 0 || jk < NP ? jk : NP - 1;
+          const DgVec<T, VW> *d = reinterpret_cast<const DgVec<T, VW> *>(sD + (jc * RS + part) * 2 * RP);
 #pragma unroll
-          for (int m = 0; m < 2; ++m) {  // Drw with Xr, then Dsw with Xs
-            const DgVec<T, VW> w = d[m * (RP / VW) + q];
+          for (int q = 0; q < RP / VW; ++q) {
 #pragma unroll
-            for (int i = 0; i < VW; i += C::RW)
-              if (q * VW + i < RI) {
+            for (int m = 0; m < 2; ++m) {  // Drw with Xr, then Dsw with Xs
+              const DgVec<T, VW> w = d[m * (RP / VW) + q];
 #pragma unroll
-                for (int f = 0; f < 3; ++f) dg_fma(&acc[f][q * VW + i], &w.v[i], y[3 * m + f]);
-              }
+              for (int i = 0; i < VW; i += C::RW)
+                if (q * VW + i < RI) {
+#pragma unroll
+                  for (int f = 0; f < 3; ++f) {
+                    T *t = &sum[f][q * VW + i];
+                    if (m == 0 && (C::PAIR || (g == 0 && k == 0)))
+                      dg_mul(t, &w.v[i], y[f]);
+                    else
+                      dg_fma(t, &w.v[i], y[3 * m + f]);
+                    if (m == 1 && C::PAIR) dg_add(&acc[f][q * VW + i], t);
+                  }
+                }
+            }
           }
         }
-      }
 #pragma unroll
-      for (int f = 0; f < 6; ++f) x[f] = xn[f];
+        for (int f = 0; f < 6; ++f) x[f] = xn[f];
+      }
+      if constexpr (!C::PAIR) {
+#pragma unroll
+        for (int f = 0; f < 3; ++f)
+#pragma unroll
+          for (int i = 0; i < RI; i += C::RW) dg_add(&acc[f][i], &sum[f][i]);
+      }
     }
     // bathymetry source at this lane's rows, then the results take the place of the fields
     asm volatile("cp.async.wait_group 1;" ::: "memory");
