@@ -22,6 +22,8 @@ __device__ int g_dg_bad;  // zero-area / clockwise triangle flag of sem_dg_geome
 
 namespace {
 
+constexpr int DG_NT = 256;  // threads of a block of k_dg_nodes
+
 __host__ __device__ constexpr int dg_np(int N) { return (N + 1) * (N + 2) / 2; }
 // Row stride of the operator block in device memory, in elements of a type of `es` bytes: an odd
 // number of 16-byte vectors, zero padded.
@@ -29,6 +31,9 @@ __host__ __device__ constexpr int dg_vw(int es) { return 16 / es; }
 __host__ __device__ constexpr int dg_ld(int N, int es) {
   return ((dg_np(N) + dg_vw(es) - 1) / dg_vw(es)) % 2 ? (dg_np(N) + dg_vw(es) - 1) / dg_vw(es) * dg_vw(es)
                                                         : ((dg_np(N) + dg_vw(es) - 1) / dg_vw(es) + 1) * dg_vw(es);
+}
+__host__ __device__ constexpr int dg_xw(int N, int es) {  // X row length: Np rounded up to whole vectors
+  return (dg_np(N) + dg_vw(es) - 1) / dg_vw(es) * dg_vw(es);
 }
 // ---------------------------------------------------------------------------------------------
 // host: operators
@@ -139,27 +144,28 @@ void vandermonde(int N, std::vector<double> &V, std::vector<double> &Vr, std::ve
 // device: volume kernel
 // ---------------------------------------------------------------------------------------------
 
-// Layout of the volume kernel.  The products are a GEMM with M = Np rows, K = 2 Np and three columns
-// (the fields) per element.  A lane owns one element and RI of its rows (RS lanes share an element):
-// it walks the nodes once, with the six flux combinations of a node in registers (nothing of X goes
-// through shared memory), and adds their products with a column of Drw and of Dsw to 3 RI
-// accumulators.  The operator columns come from shared memory 16 bytes at a time, one load for 3 x 4
-// products; FP32 products run two rows to an instruction (FFMA2: the scalar FMA rate at half the
-// issue slots).  A warp stages the fields of its WE elements by asynchronous copies, one batch ahead,
-// and its results leave through the same buffer; warps are independent of one another.
+// Layout of the volume kernel for meshes that fill the chip (k_dg_nodes below for smaller ones, see
+// dg_rule).  The products are a GEMM with M = Np rows, K = 2 Np and three columns (the fields) per element.  A
+// lane owns one element and RI of its rows (RS lanes share an element): it walks the nodes once, with the
+// six flux combinations of a node in registers (nothing of X goes through shared memory), and adds their
+// products with a column of Drw and of Dsw to 3 RI sums.  The operator columns come from shared memory
+// 16 bytes at a time, one load for 3 x 4 products; FP32 products run two rows to an instruction (FFMA2: the
+// scalar FMA rate at half the issue slots).  A warp stages the fields of its WE elements by asynchronous
+// copies, one batch ahead, and its results leave through the same buffer; warps are independent of one
+// another.
 //
 // Rounding: the products of SG * RS nodes are summed on their own and then added to the output, so that most
-// roundings happen at a fraction of its size (one addition in 8 to 14 products).  RMS error against FP64,
+// roundings happen at a fraction of its size (one addition in 8 to 16 products).  RMS error against FP64,
 // FP32, of each node's pair of products added to the output / one chain of all products / these groups:
 // N = 3 8.76e-8 / 9.12e-8 / 8.22e-8, 5 1.05e-7 / 1.13e-7 / 9.2e-8, 7 1.40e-7 / 1.48e-7 / 1.22e-7, 8 1.72e-7 /
-// 1.82e-7 / 1.58e-7.  At N = 1 and 2 (3 and 6 nodes) groups gain nothing: pairs there.
+// 1.82e-7 / 1.58e-7.  At N = 1 (3 nodes) groups gain nothing, and in FP32 at N = 2 they take registers: pairs there.
 //
-// What bounds it at N = 7, FP32: the operator loads (each returns 512 bytes to registers, four
-// cycles of the SM's shared-memory path, for 12 FMA cycles per scheduler) and the FMA pipe, half
-// busy; with the products left out the copies alone take 48 us of the 99 us.  212,800 triangles,
-// before (one thread per node of 1 to 3 elements, X in shared memory) / now, L2 flushed: FP32
-// N = 1..8 13 / 11, 23 / 16, 35 / 21, 81 / 33, 130 / 48, 111 / 74, 163 / 99, 326 / 150 us, FP64 N = 4
-// 1012 / 691, 8 8697 / 5199 us (the FP64 pipe: 4640 us for the products alone).
+// What bounds it at N = 7, FP32: the operator loads (each returns 512 bytes to registers, four cycles of the
+// SM's shared-memory path, for 12 FMA cycles per scheduler) and the FMA pipe, half busy; with the products
+// left out the copies alone take 48 us of the 95 us.  212,552 triangles, k_dg_nodes / this kernel, caches warm: FP32
+// N = 1..8 7.4 / 5.6, 17 / 8.6, 28 / 14, 79 / 26, 135 / 42, 109 / 67, 154 / 95, 319 / 147 us; FP64 N = 3..8 387 / 353,
+// 822 / 721, 1508 / 1374, 2478 / 2224, 3977 / 3537, 6966 / 5759 us (the FP64 pipe: 4640 us at N = 8 for the products
+// alone).
 template <typename T, int N, int RS_>
 struct DgCfg {
   static constexpr int NP = dg_np(N), VW = dg_vw(sizeof(T)), RS = RS_;
@@ -167,9 +173,14 @@ struct DgCfg {
   static constexpr int RW = sizeof(T) == 4 ? 2 : 1;         // rows per product instruction
   static constexpr int RI = ((NP + RS - 1) / RS + RW - 1) / RW * RW;  // rows per lane
   static constexpr int RP = (RI + VW - 1) / VW * VW;        // row stride of an operator column
-  static constexpr bool PAIR = N <= 2;                      // a node's two products join the sum by themselves
+  static constexpr bool PAIR = N == 1 || (N == 2 && sizeof(T) == 4);  // a node's two products join the sum by themselves
   // else the products of SG * RS nodes do (a divisor of Np where there is one near)
-  static constexpr int SG = PAIR || RS == 4 ? 1 : RS == 2 ? (N == 6 ? 2 : 3) : N == 5 ? 7 : 5;
+  static constexpr int SG = PAIR                ? 1
+                            : RS == 4           ? (sizeof(T) == 8 && N >= 4 ? 2 : 1)
+                            : N == 2            ? 2 / RS
+                            : RS == 2           ? (N == 6 ? 2 : 3)
+                            : N == 5            ? 7
+                                                : 5;
   static constexpr int QW = WE * 3 * NP, BW = WE * 2 * NP;  // field and bathymetry values of a batch
   static constexpr int PW = 2 * QW + BW;                    // values staged per warp (fields twice)
   static constexpr int DW = NP * RS * 2 * RP;               // operator values per block
@@ -205,8 +216,8 @@ __device__ __forceinline__ void dg_add(double *a, const double *b) { *a += *b; }
 
 // 1 / h: one Newton-Raphson step on the hardware's approximation in its fused form, r + r (1 - h r) (Markstein,
 // IBM J. Res. Dev. 34, 1990), within a unit in the last place of the quotient.  A division's branch would
-// keep the fluxes of the next node apart from the products of this one (212,800 triangles, FP32, N = 7: 107
-// against 99 us).  The approximation itself is kept where the step has no meaning: h zero, infinite or so small
+// keep the fluxes of the next node apart from the products of this one (212,552 triangles, FP32, N = 7: 103
+// against 95 us).  The approximation itself is kept where the step has no meaning: h zero, infinite or so small
 // that its reciprocal overflows (the error is then NaN or infinite).
 __device__ __forceinline__ float dg_reciprocal(float h) {
   float r;
@@ -324,7 +335,12 @@ __global__ void __launch_bounds__(32 * DgCfg<T, N, RS_>::W)
                       dg_mul(t, &w.v[i], y[f]);
                     else
                       dg_fma(t, &w.v[i], y[3 * m + f]);
-                    if (m == 1 && C::PAIR) dg_add(&acc[f][q * VW + i], t);
+                    if (m == 1 && C::PAIR) {
+                      if (sizeof(T) == 8 && g == 0 && k == 0 && j0 == 0)
+                        for (int r = 0; r < C::RW; ++r) acc[f][q * VW + i + r] = t[r];
+                      else
+                        dg_add(&acc[f][q * VW + i], t);
+                    }
                   }
                 }
             }
@@ -334,10 +350,17 @@ __global__ void __launch_bounds__(32 * DgCfg<T, N, RS_>::W)
         for (int f = 0; f < 6; ++f) x[f] = xn[f];
       }
       if constexpr (!C::PAIR) {
+        if (sizeof(T) == 8 && j0 == 0) {  // (an FP64 addition less)
 #pragma unroll
-        for (int f = 0; f < 3; ++f)
+          for (int f = 0; f < 3; ++f)
 #pragma unroll
-          for (int i = 0; i < RI; i += C::RW) dg_add(&acc[f][i], &sum[f][i]);
+            for (int i = 0; i < RI; ++i) acc[f][i] = sum[f][i];
+        } else {
+#pragma unroll
+          for (int f = 0; f < 3; ++f)
+#pragma unroll
+            for (int i = 0; i < RI; i += C::RW) dg_add(&acc[f][i], &sum[f][i]);
+        }
       }
     }
     // bathymetry source at this lane's rows, then the results take the place of the fields
@@ -389,6 +412,116 @@ __global__ void __launch_bounds__(32 * DgCfg<T, N, RS_>::W)
   }
 }
 
+// The volume kernel for small meshes: one thread per element node.  A block takes batches of
+// floor(256 / Np) groups of ET elements and stays resident over many batches; the operators (rows zero
+// padded to an odd number of 16-byte vectors, so that threads on consecutive rows hit distinct banks) and
+// the batch's Xr, Xs sit in shared memory and are read 16 bytes at a time (X as a broadcast).
+// Elements per thread: with ET > 1 every operator vector serves ET elements (212,800 triangles: ET = 2 1.2x
+// over 1 at N = 6..8, slower at N = 2; ET = 3 a further 5% at N = 7 and 8.5% at N = 8; ET = 4 slower); FP64 keeps
+// 1 (its FMA pipe is the bound, and its shared memory would not fit).
+__host__ __device__ constexpr int dg_et(int N, int es) { return es == 4 && N >= 7 ? 3 : es == 4 && N >= 3 ? 2 : 1; }
+
+template <typename T, int N>
+__global__ void __launch_bounds__(DG_NT) k_dg_nodes(int64_t E, T g, const T *__restrict__ ops,
+                                                     const T *__restrict__ Q, const T *__restrict__ Bxy,
+                                                     const T *__restrict__ geo, T *__restrict__ rhs) {
+  constexpr int NP = dg_np(N), LD = dg_ld(N, sizeof(T)), XW = dg_xw(N, sizeof(T));
+  constexpr int ET = dg_et(N, sizeof(T)), EG = DG_NT / NP, EB = EG * ET;  // groups, elements per batch
+  constexpr int VW = dg_vw(sizeof(T)), NV = XW / VW;  // 16-byte vectors per row
+  __shared__ alignas(16) T sD[2 * NP * LD];
+  __shared__ alignas(16) T sX[EB][6][XW];
+  const int tid = threadIdx.x;
+  for (int q = tid; q < 2 * NP * LD; q += DG_NT) sD[q] = ops[q];
+  // zero the padding of the X rows (it meets the zero padding of the operator rows)
+  if constexpr (XW > NP) {
+    for (int q = tid; q < EB * 6 * (XW - NP); q += DG_NT) {
+      const int row = q / (XW - NP);
+      sX[row / 6][row % 6][NP + q % (XW - NP)] = T(0);
+    }
+  }
+  const int el = tid / NP, i = tid - el * NP;  // group (ET consecutive elements of a batch), node
+  const bool grp = el < EG;
+  const DgVec<T, VW> *dr = reinterpret_cast<const DgVec<T, VW> *>(sD + i * LD);
+  const DgVec<T, VW> *ds = reinterpret_cast<const DgVec<T, VW> *>(sD + NP * LD + i * LD);
+  const DgVec<T, VW> *x0 = reinterpret_cast<const DgVec<T, VW> *>(&sX[grp ? el * ET : 0][0][0]);
+  constexpr int XS = 6 * NV;  // vectors per element in sX
+  // persistent blocks: the operators are loaded once per block, batches of EB elements follow
+  const int64_t nbatch = (E + EB - 1) / EB;
+  for (int64_t batch = blockIdx.x; batch < nbatch; batch += gridDim.x) {
+    const int64_t e0 = batch * EB + (int64_t)el * ET;
+    T h[ET], bx[ET], by[ET];
+#pragma unroll
+    for (int t = 0; t < ET; ++t) {
+      const int64_t e = e0 + t;
+      h[t] = T(1), bx[t] = T(0), by[t] = T(0);
+      if (grp && e < E) {
+        const T *q = Q + e * 3 * NP + i;
+        h[t] = q[0];
+        const T hu = q[NP], hv = q[2 * NP];
+        bx[t] = Bxy[e * 2 * NP + i];
+        by[t] = Bxy[e * 2 * NP + NP + i];
+        const T rx = geo[e * 4 + 0], ry = geo[e * 4 + 1], sx = geo[e * 4 + 2], sy = geo[e * 4 + 3];
+        const T ih = T(1) / h[t], u = hu * ih, v = hv * ih, p = T(0.5) * g * h[t] * h[t];
+        const T F0 = hu, F1 = hu * u + p, F2 = hu * v;
+        const T G0 = hv, G1 = hv * u, G2 = hv * v + p;
+        T(*X)[XW] = sX[el * ET + t];
+        X[0][i] = rx * F0 + ry * G0;
+        X[1][i] = rx * F1 + ry * G1;
+        X[2][i] = rx * F2 + ry * G2;
+        X[3][i] = sx * F0 + sy * G0;
+        X[4][i] = sx * F1 + sy * G1;
+        X[5][i] = sx * F2 + sy * G2;
+      }
+    }
+    __syncthreads();
+    if (grp && e0 < E) {
+      // 16-byte loads: one operator vector serves three fields of ET elements; each X vector is the
+      // same for every thread of the element (a broadcast)
+      T a[ET][3];
+#pragma unroll
+      for (int t = 0; t < ET; ++t) a[t][0] = a[t][1] = a[t][2] = T(0);
+#pragma unroll
+      for (int jv = 0; jv < NV; ++jv) {
+        const DgVec<T, VW> wr = dr[jv], ws = ds[jv];
+#pragma unroll
+        for (int t = 0; t < ET; ++t) {
+          const DgVec<T, VW> *xt = x0 + t * XS;
+          const DgVec<T, VW> r0 = xt[0 * NV + jv], r1 = xt[1 * NV + jv], r2 = xt[2 * NV + jv];
+          const DgVec<T, VW> s0 = xt[3 * NV + jv], s1 = xt[4 * NV + jv], s2 = xt[5 * NV + jv];
+          // a vector's products are summed on their own (N = 1: a node's), as in k_dg_volume
+          T p0 = T(0), p1 = T(0), p2 = T(0);
+#pragma unroll
+          for (int k = 0; k < VW; ++k) {
+            if (N == 1 || k == 0) {
+              p0 = wr.v[k] * r0.v[k], p1 = wr.v[k] * r1.v[k], p2 = wr.v[k] * r2.v[k];
+            } else {
+              p0 += wr.v[k] * r0.v[k], p1 += wr.v[k] * r1.v[k], p2 += wr.v[k] * r2.v[k];
+            }
+            p0 += ws.v[k] * s0.v[k], p1 += ws.v[k] * s1.v[k], p2 += ws.v[k] * s2.v[k];
+            if (N == 1 || k == VW - 1) {
+              if (jv == 0 && (N > 1 || k == 0))
+                a[t][0] = p0, a[t][1] = p1, a[t][2] = p2;
+              else
+                a[t][0] += p0, a[t][1] += p1, a[t][2] += p2;
+            }
+          }
+        }
+      }
+#pragma unroll
+      for (int t = 0; t < ET; ++t) {
+        const int64_t e = e0 + t;
+        if (e < E) {
+          T *o = rhs + e * 3 * NP + i;
+          o[0] = a[t][0];
+          o[NP] = a[t][1] - g * h[t] * bx[t];
+          o[2 * NP] = a[t][2] - g * h[t] * by[t];
+        }
+      }
+    }
+    __syncthreads();  // the next batch overwrites sX
+  }
+}
+
 // rx, ry, sx, sy of each triangle: the inverse of [[x_r, x_s], [y_r, y_s]] with x_r = (x2 - x1)/2,
 // x_s = (x3 - x1)/2 (and y alike); bad is set when the Jacobian is not positive
 template <typename T>
@@ -407,7 +540,7 @@ __global__ void k_dg_geometry(int64_t E, const double *__restrict__ v, T *__rest
 }
 
 template <typename T, int N, int RS>
-sem_status launch_dg_rs(int64_t E, double g, const void *ops, const void *Q, const void *Bxy, const void *geo,
+sem_status launch_dg_lanes(int64_t E, double g, const void *ops, const void *Q, const void *Bxy, const void *geo,
                         void *rhs, int sms, cudaStream_t s) {
   using C = DgCfg<T, N, RS>;
   static std::atomic<unsigned long long> attr_done;
@@ -426,20 +559,74 @@ sem_status launch_dg_rs(int64_t E, double g, const void *ops, const void *Q, con
   return SEM_OK;
 }
 
-// Lanes per element on a mesh that fills the device: one while 3 Np accumulators fit in registers
-// beside the rest (measured at 212,800 triangles, FP32, 1 / 2 / 4 lanes: N = 4 32 / 38 / 36 us,
-// 5 48 / 52 / 56, 6 79 / 70 / 79, 7 107 / 99 / 99; FP64, 1 / 2 lanes: N = 4 674 / 855, 5 1340 / 1424).
-// Below four warps per SM, four lanes: a few elements then spread over more schedulers (FP64, 4000
-// triangles, 1 or 2 / 4 lanes: N = 3 37 / 17 us, 8 265 / 137).
+template <typename T, int N>
+sem_status launch_dg_nodes(int64_t E, double g, const void *ops, const void *Q, const void *Bxy, const void *geo,
+                           void *rhs, int sms, cudaStream_t s) {
+  constexpr int EB = DG_NT / dg_np(N) * dg_et(N, sizeof(T));
+  int per_sm = 0;
+  SEM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_dg_nodes<T, N>, DG_NT, 0));
+  const int64_t batches = (E + EB - 1) / EB, resident = (int64_t)sms * (per_sm > 0 ? per_sm : 1);
+  const int64_t blocks = batches < resident ? batches : resident;
+  k_dg_nodes<T, N><<<(unsigned)blocks, DG_NT, 0, s>>>(
+      E, (T)g, static_cast<const T *>(ops), static_cast<const T *>(Q), static_cast<const T *>(Bxy),
+      static_cast<const T *>(geo), static_cast<T *>(rhs));
+  SEM_CUDA_TRY(cudaGetLastError());
+  return SEM_OK;
+}
+
+// Which kernel a mesh of E triangles takes, by triangles per SM: below `a` one thread per node, below `b` `f1`
+// lanes per element, from there `f2` lanes (0: one thread per node).  A warp of the lane form holds 8 to 32
+// elements, so that a small mesh leaves schedulers without a warp (FP64 above all, whose pipe belongs to a
+// scheduler); one thread per node spreads it.  More lanes per element lie between.  Measured with the
+// caches warm, us for one thread per node | 1 / 2 / 4 lanes:
+//   FP32, 3200 triangles     N = 2 2.1 | 2.6 / 2.6 / 2.6   4 3.6 | 4.0 / 3.9 / 3.4    7 6.4 | - / 8.0 / 8.3
+//         8192               N = 3 3.4 | 2.9 / 3.5 / 3.7   5 8.2 | 5.6 / 5.6 / 5.6    7 9.4 | - / 8.5 / 8.6
+//         33800              N = 1 2.6 | 2.7 / 2.9 / 3.2   4 13.5 | 6.0 / 6.6 / 8.0   8 53 | - / 30 / 33
+//         212,552            N = 1 7.4 | 5.6 / 8.2 / 11.5  6 106 | 73 / 67 / 72       8 320 | 313 / 147 / 159
+//   FP64, 800                N = 1 5.9 | 8.1 / 7.3 / 4.2   4 11.8 | 65 / 39 / 21.4    7 23 | - / 159 / 86
+//         3200               N = 3 8.5 | 34 / 19 / 14.4    5 28 | - / 67 / 42         7 82 | - / 159 / 86
+//         15488              N = 3 36 | 35 / 31 / 40       5 118 | - / 113 / 135      8 525 | - / 524 / 483
+//         45000              N = 2 40 | 45 / 47 / 68       4 179 | 175 / 183 / 190    8 1499 | - / 1318 / 1332
+struct DgRule {
+  int a, f1, b, f2;
+};
+template <typename T>
+__host__ __device__ constexpr DgRule dg_rule(int N) {
+  if (sizeof(T) == 4)
+    return N == 1   ? DgRule{260, 1, 0, 1}
+           : N == 2 ? DgRule{85, 1, 0, 1}
+           : N == 3 ? DgRule{50, 1, 0, 1}
+           : N == 4 ? DgRule{0, 4, 50, 1}
+           : N == 5 ? DgRule{26, 1, 0, 1}
+           : N == 6 ? DgRule{40, 2, 0, 2}
+           : N == 7 ? DgRule{50, 2, 0, 2}
+                    : DgRule{25, 2, 0, 2};
+  return N == 1   ? DgRule{0, 4, 50, 0}
+         : N == 2 ? DgRule{0, 0, 0, 0}
+         : N == 3 ? DgRule{145, 1, 0, 1}
+         : N == 4 ? DgRule{46, 4, 115, 1}
+         : N == 5 ? DgRule{145, 2, 0, 2}
+                  : DgRule{25, 4, 0, 4};
+}
+
 template <typename T, int N>
 sem_status launch_dg(int64_t E, double g, const void *ops, const void *Q, const void *Bxy, const void *geo,
                      void *rhs, cudaStream_t s) {
-  constexpr int RS = N >= 6 ? 2 : 1;
+  constexpr DgRule R = dg_rule<T>(N);
   int dev = 0, sms = 0;
   SEM_CUDA_TRY(cudaGetDevice(&dev));
   SEM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  if (E < (int64_t)sms * 4 * (32 / RS)) return launch_dg_rs<T, N, 4>(E, g, ops, Q, Bxy, geo, rhs, sms, s);
-  return launch_dg_rs<T, N, RS>(E, g, ops, Q, Bxy, geo, rhs, sms, s);
+  if constexpr (R.a > 0 || R.f2 == 0) {
+    if (E < (int64_t)sms * R.a || (R.f2 == 0 && E >= (int64_t)sms * R.b))
+      return launch_dg_nodes<T, N>(E, g, ops, Q, Bxy, geo, rhs, sms, s);
+  }
+  if constexpr (R.f1 > 0 && R.b > 0) {
+    if (R.f2 == 0 || E < (int64_t)sms * R.b) return launch_dg_lanes<T, N, R.f1>(E, g, ops, Q, Bxy, geo, rhs, sms, s);
+  }
+  if constexpr (R.f2 > 0)
+    return launch_dg_lanes<T, N, R.f2>(E, g, ops, Q, Bxy, geo, rhs, sms, s);
+  else
+    return SEM_OK;  // not reached
 }
 
 template <typename T>
