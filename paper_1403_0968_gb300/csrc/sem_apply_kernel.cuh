@@ -272,16 +272,16 @@ __host__ __device__ constexpr size_t apply_red_off() {
          16 * 16;
 }
 
-// bytes of the reduction slots: 32 doubles (batched per-element sums) or one value per thread
-template <int NP, typename T, int EB>
+// bytes of the reduction slots: 32 doubles (batched per-element sums) or, for a solve's sum, one value per thread
+template <int NP, typename T, int EB, bool DOT>
 __host__ __device__ constexpr size_t apply_red_size() {
-  constexpr size_t per_thread = ((size_t)ApplyCfg<NP, EB>::NT * sizeof(T) + 15) / 16 * 16;
+  constexpr size_t per_thread = !DOT ? 0 : ((size_t)ApplyCfg<NP, EB>::NT * sizeof(T) + 15) / 16 * 16;
   return per_thread > 32 * 8 ? per_thread : 32 * 8;
 }
 
-template <int NP, typename T, int EB, bool STAGE, typename TG = T>
+template <int NP, typename T, int EB, bool STAGE, typename TG = T, bool DOT = true>
 __host__ __device__ constexpr size_t apply_smem() {
-  return apply_red_off<NP, T, EB, STAGE, TG>() + apply_red_size<NP, T, EB>() + 16;
+  return apply_red_off<NP, T, EB, STAGE, TG>() + apply_red_size<NP, T, EB, DOT>() + 16;
 }
 
 // BOXM: structured box numbering with no mask array (bc NONE or BOX): global ids and Dirichlet
@@ -289,8 +289,18 @@ __host__ __device__ constexpr size_t apply_smem() {
 // Minimum resident blocks the FP32 kernel's registers are held to at high order, where one
 // element per block otherwise leaves one or two blocks per SM; 0 = no floor (an explicit 1 lets the
 // compiler take more registers).
-template <typename T>
+// Plain applies with explicit numbering take registers for the node ids.  Where the compiler gave an order fewer
+// blocks per SM for them than a box has, these are asked for: on the fly, us at about 7e6 nodes with the
+// floor / without: N = 5 142 / 160, 7 128 / 160, 9 166 / 197, 11 198 / 242; BF16 N = 11 149 / 168.
+template <typename T, typename TG, bool PLAIN_GLO>
 __host__ __device__ constexpr int apply_min_blocks(int NP, int EB) {
+  if (PLAIN_GLO && is_otf<TG>() && EB == apply_eb_default(NP)) {
+    if (NP == 5 || NP == 6) return 7;
+    if (NP == 10) return 6;
+    if (NP == 12) return 4;
+  }
+  if (PLAIN_GLO && is_otf<TG>() && NP == 8 && EB == 1) return 14;
+  if (PLAIN_GLO && sizeof(T) == 4 && NP == 12 && EB == 1) return 6;
   return (sizeof(T) == 4 && EB == 1 && NP >= 13 && NP <= 15) ? 2 : 0;  // measured: +15-35% at N = 12..14
 }
 
@@ -315,27 +325,33 @@ __host__ __device__ constexpr bool apply_prefetch(int NP) {
 
 // Packed line products (line_eo).  GDOF/s at 8e6 nodes, scalar / packed: FP32 factors N = 3 121 / 116, 5
 // 111 / 105, 7 120 / 122, 10 113 / 115; BF16 7 138 / 144, 8 133 / 151, 9 125 / 143; on the fly 4 118 / 129,
-// 5 114 / 126, 7 149 / 155, 9 125 / 118, 10 145 / 151.
+// 5 114 / 126, 7 149 / 155, 9 125 / 118, 10 145 / 151; us at 2.5e6 nodes 1 23.3 / 23.1, 2 23.8 / 23.7, 3 19.6 / 19.3,
+// 6 24.9 / 23.0, 8 23.4 / 22.9, 11 21.1 / 20.7.
 template <typename T, typename TG>
 __host__ __device__ constexpr bool apply_packed(int NP) {
   return sizeof(T) == 4 && (is_otf<TG>() ? NP != 10 : sizeof(TG) == 2 || NP >= 7);
 }
 
-// TG: storage type of the factors (T, or BF16 with T = float: half the factor traffic)
-template <int NP, typename T, int EB_, bool STAGE, bool BOXM, typename TG = T>
-__global__ void __launch_bounds__(ApplyCfg<NP, EB_>::NT, apply_min_blocks<T>(NP, EB_))
+// TG: storage type of the factors (T, or BF16 with T = float: half the factor traffic).
+// DOT: with the sum of a CG step, run when P.partials is set.  Explicit numbering has plain applies without that
+// code, with scalar line products and without held factors (PREF): on top of its node ids the registers of
+// any of the three cost more than they gave.  Explicit numbering at about 7e6 nodes, us, with all three / without:
+// FP32 N = 4 129 / 95, 5 158 / 118, 9 174 / 157; BF16 N = 8 128 / 104, 11 181 / 168; on the fly N = 6 199 / 173, 8 237 /
+// 150, 11 257 / 242; FP64 N = 15 1327 / 1270.
+template <int NP, typename T, int EB_, bool STAGE, bool BOXM, typename TG, bool DOT>
+__global__ void __launch_bounds__(ApplyCfg<NP, EB_>::NT, apply_min_blocks<T, TG, !BOXM && !DOT>(NP, EB_))
     k_apply(const ApplyParams<T, NP> P) {
   using C = ApplyCfg<NP, EB_>;
   constexpr int N = NP - 1, NP2 = C::NP2, NP3 = C::NP3, EB = C::EB, NT = C::NT, RS = C::RS, PS = C::PS,
                 BUF = C::BUF, GS = factor_stride<NP, TG>();
   extern __shared__ __align__(128) unsigned char smem_raw[];
   constexpr size_t RED_OFF = apply_red_off<NP, T, EB_, STAGE, TG>();
-  constexpr bool PK = apply_packed<T, TG>(NP);
+  constexpr bool PK = BOXM && apply_packed<T, TG>(NP);
   static_assert(RED_OFF % 16 == 0 && ((STAGE ? EB * GS : 0) * sizeof(TG)) % 16 == 0, "shared-memory alignment");
   TG *sG = reinterpret_cast<TG *>(smem_raw);  // TMA destination: 16-byte aligned at offset 0
   T *sbuf = reinterpret_cast<T *>(smem_raw + (STAGE ? EB * GS * sizeof(TG) : 0));
   double *s_red = reinterpret_cast<double *>(smem_raw + RED_OFF);
-  uint64_t *bar = reinterpret_cast<uint64_t *>(smem_raw + RED_OFF + apply_red_size<NP, T, EB_>());
+  uint64_t *bar = reinterpret_cast<uint64_t *>(smem_raw + RED_OFF + apply_red_size<NP, T, EB_, DOT>());
 
   const int tid = threadIdx.x;
   const int es = tid / NP2, t2 = tid - es * NP2, a = t2 % NP, b = t2 / NP;
@@ -354,7 +370,7 @@ __global__ void __launch_bounds__(ApplyCfg<NP, EB_>::NT, apply_min_blocks<T>(NP,
   }
   // inside a solve: the kernel before this one has to be complete (the factors, asked for above, depend
   // on no kernel of the solve); nothing to do once the iteration has stopped
-  if (P.scal) {
+  if (DOT && P.scal) {
     dependent_wait();
     if (P.scal->converged || P.scal->breakdown) {
       if constexpr (STAGE) {
@@ -404,7 +420,7 @@ __global__ void __launch_bounds__(ApplyCfg<NP, EB_>::NT, apply_min_blocks<T>(NP,
       if (__syncthreads_and(skip)) return;  // every element of this block is finished
     }
   }
-  constexpr bool PREF = apply_prefetch<T, TG, STAGE>(NP);
+  constexpr bool PREF = BOXM && apply_prefetch<T, TG, STAGE>(NP);
   TG gpre[PREF ? 6 * NP : 1];
   if constexpr (PREF) {
     const TG *Ge = c_Gf + (active ? el : 0) * P.gs + t2;
@@ -635,7 +651,7 @@ __global__ void __launch_bounds__(ApplyCfg<NP, EB_>::NT, apply_min_blocks<T>(NP,
   // Optional arrays are tested through their own pointers, here and for kappa above: a pointer that was
   // offset first ("q ? q + i : nullptr") and then tested was dereferenced with q null in the FP64 form
   // of this kernel, where a build of the same source for the host is clean.
-  if (P.partials) {
+  if (DOT && P.partials) {
     // p^T A p and the CG step length: one warp adds the block's terms and publishes them before its
     // scatter, so that its fences have no writes to wait for and the other warps do not wait at all
     T dotp = T(0);
@@ -660,9 +676,11 @@ __global__ void __launch_bounds__(ApplyCfg<NP, EB_>::NT, apply_min_blocks<T>(NP,
       if (!((dirbits >> k) & 1u)) scatter(k, yc[k]);
     return;
   }
+  if (!BOXM && !active) return;
   T dotp = T(0);
 #pragma unroll
   for (int k = 0; k < NP; ++k) {
+    if (!BOXM && ((dirbits >> k) & 1u)) continue;
     const int q = k * PS + b * RS + a;
     T yk = yc[k] + sr[q] + ss[q];
     if (c_wJa && active) yk += c_wJa[el * NP3 + t2 + NP2 * k] * uc[k];
@@ -700,26 +718,25 @@ static sem_status launch_apply_v(const ApplyParams<T, NP> &p, cudaStream_t s) {
   using C = ApplyCfg<NP, EB>;
   const unsigned grid = (unsigned)((p.E + C::EB - 1) / C::EB);
   if (p.partials && grid > SEM_MAX_PARTIALS) return sem_fail(SEM_ERR_INVALID, "too many elements for fused dot");
-  constexpr size_t smem = apply_smem<NP, T, EB, STAGE, TG>();
-  static_assert(smem <= SEM_MAX_SMEM_PER_BLOCK, "apply variant exceeds the shared memory of a block");
+  static_assert(apply_smem<NP, T, EB, STAGE, TG>() <= SEM_MAX_SMEM_PER_BLOCK,
+                "apply variant exceeds the shared memory of a block");
   const bool boxm = p.glo == nullptr && p.bc != SEM_BC_MASK;
-  static std::atomic<unsigned long long> attr_done[2];
-  {
-    const cudaError_t e = boxm ? set_smem_limit_once(k_apply<NP, T, EB, STAGE, true, TG>, smem, attr_done[1])
-                               : set_smem_limit_once(k_apply<NP, T, EB, STAGE, false, TG>, smem, attr_done[0]);
-    if (e != cudaSuccess) return sem_fail(SEM_ERR_CUDA, std::string("apply smem attribute: ") + cudaGetErrorString(e));
-  }
-  cudaError_t e;
-  if (p.scal) {  // a step of a solve
-    e = boxm ? launch_dependent(k_apply<NP, T, EB, STAGE, true, TG>, grid, C::NT, smem, s, p)
-             : launch_dependent(k_apply<NP, T, EB, STAGE, false, TG>, grid, C::NT, smem, s, p);
-  } else {
-    if (boxm)
-      k_apply<NP, T, EB, STAGE, true, TG><<<grid, C::NT, smem, s>>>(p);
-    else
-      k_apply<NP, T, EB, STAGE, false, TG><<<grid, C::NT, smem, s>>>(p);
-    e = cudaGetLastError();
-  }
+  static std::atomic<unsigned long long> attr_done[4];
+  auto launch = [&](auto *kernel, size_t smem, std::atomic<unsigned long long> &done) {
+    cudaError_t e = set_smem_limit_once(kernel, smem, done);
+    if (e != cudaSuccess) return e;
+    if (p.scal) return launch_dependent(kernel, grid, C::NT, smem, s, p);  // a step of a solve
+    kernel<<<grid, C::NT, smem, s>>>(p);
+    return cudaGetLastError();
+  };
+  constexpr size_t plain = apply_smem<NP, T, EB, STAGE, TG, false>(), dot = apply_smem<NP, T, EB, STAGE, TG, true>();
+  // on boxes one kernel serves plain applies too, except where the code of the sum makes registers spill (on the
+  // fly, 14^3 and 13^3 elements, in one / apart: N = 13 131 / 114 us, 14 156 / 139)
+  constexpr bool SPLIT = is_otf<TG>() && (NP == 14 || NP == 15);
+  const cudaError_t e = boxm && (p.scal || !SPLIT) ? launch(k_apply<NP, T, EB, STAGE, true, TG, true>, dot, attr_done[0])
+                        : boxm                     ? launch(k_apply<NP, T, EB, STAGE, true, TG, !SPLIT>, SPLIT ? plain : dot, attr_done[3])
+                        : p.scal ? launch(k_apply<NP, T, EB, STAGE, false, TG, true>, dot, attr_done[1])
+                                 : launch(k_apply<NP, T, EB, STAGE, false, TG, false>, plain, attr_done[2]);
   if (e != cudaSuccess) return sem_fail(SEM_ERR_CUDA, std::string("apply launch: ") + cudaGetErrorString(e));
   return SEM_OK;
 }
@@ -743,11 +760,11 @@ __host__ __device__ constexpr size_t pipe_smem();
 // nodes, variants 0 / 1 / 3): FP32 N = 2 116 / 109 / 113, 3 108 / 121 / 111, 5 107 / 111 / 110, 6 110 / 93 /
 // 113, 7 122 / 100 / 116, 15 56 / 56 / 56 (the former choice there, 2: 49); BF16 N = 2 141 / 120 / 136, 3
 // 145 / 127 / 145, 5 130 / 108 / 114, 6 135 / 105 / 140, 7 144 / 106 / 139, 15 74 / 58 / 74; on the fly
-// (no factor block: 0 = 1) N = 3 139 / 139, 5 126 / 97, 6 120 / 116, 7 147 / 155 (variants 1 / 3).  FP64
-// takes 1 (k_apply_cols where it is the faster one).
+// (no factor block: 0 = 1) N = 3 139 / 139, 5 126 / 97, 6 120 / 116, 7 147 / 155 (variants 1 / 3), with explicit
+// numbering N = 6 172 / 139 us at 27^3 elements.  FP64 takes 1 (k_apply_cols where it is the faster one).
 template <typename T, typename TG>
-__host__ __device__ constexpr int apply_auto_variant(int NP) {
-  return is_otf<TG>() ? (NP == 4 || NP == 8 ? 3 : 1)
+__host__ __device__ constexpr int apply_auto_variant(int NP, bool general) {
+  return is_otf<TG>() ? (NP == 4 || NP == 8 || (general && NP == 7) ? 3 : 1)
          : sizeof(T) == 8 ? 1
          : NP == 7 ? 3
          : sizeof(TG) == 2 ? 0
@@ -922,7 +939,7 @@ static sem_status launch_apply_cols(const ApplyParams<double, NP> &p, cudaStream
 
 template <int NP, typename T, typename TG = T>
 static sem_status launch_apply_np(const ApplyParams<T, NP> &p, int variant, cudaStream_t s) {
-  if (variant < 0) variant = apply_auto_variant<T, TG>(NP);
+  if (variant < 0) variant = apply_auto_variant<T, TG>(NP, p.glo != nullptr || p.bc == SEM_BC_MASK);
   if constexpr (std::is_same<T, double>::value && NP >= 4 && NP <= 15 && NP != 11) {
     // (a solve's fused sum takes one partial per block; beyond that many elements, k_apply's larger blocks)
     if (variant == 1 && p.batch == nullptr && apply_cols(NP, p.E) && (!p.partials || p.E <= SEM_MAX_PARTIALS))
