@@ -234,11 +234,16 @@ struct EmuParams {
   EvenOdd<NP> EO;
 };
 
+// Forms of the kernel by problem size (emu_form): fuller blocks for a chip full of them, one or two elements
+// per block without register floors, and the same in scalar arithmetic.
+enum EmuForm { EMU_FULL, EMU_SMALL, EMU_SCALAR };
+
 // Whether an order runs its line products and factor scaling in packed form (DOT: with the fused
 // reduction of a CG step, whose registers come on top).  Measured, GDOF/s at 1.6e7 nodes, scalar /
 // packed: plain N = 2 59 / 57, 4 52 / 51, 10 32 / 30, 7 42 / 44.5, 11 20.6 / 24.6, 15 17 / 26; DOT
 // N = 5 43 / 37, 6 36 / 36, 7 42 / 40, 8 35.5 / 28, 9 27 / 30, 15 14.5 / 21.
-__host__ __device__ constexpr bool emu_packed(int NP, bool dot) {
+__host__ __device__ constexpr bool emu_packed(int NP, bool dot, EmuForm form) {
+  if (form == EMU_SCALAR) return false;
   return NP == 4 || NP == 10 || NP >= 12 || (!dot && NP >= 6 && NP <= 9);
 }
 // whether the even and odd parts of a line are formed together too (N = 15 one after the other: 26 GDOF/s
@@ -312,13 +317,13 @@ __device__ __forceinline__ void df_line(const EmuParams<NP> &P, const float2 (&v
 __host__ __device__ constexpr int emu_eb_staged(int NP) {
   return NP <= 2 ? 32 : NP == 3 ? 14 : NP == 4 ? 8 : NP == 5 ? 5 : NP == 6 ? 3 : NP <= 8 ? 2 : 1;
 }
-__host__ __device__ constexpr int emu_eb(int NP, bool small) {
-  return small ? emu_eb_staged(NP) : NP == 6 ? 7 : NP == 7 ? 5 : (NP == 9 || NP == 10) ? 3 : NP == 12 ? 2 : emu_eb_staged(NP);
+__host__ __device__ constexpr int emu_eb(int NP, EmuForm form) {
+  return form != EMU_FULL ? emu_eb_staged(NP) : NP == 6 ? 7 : NP == 7 ? 5 : (NP == 9 || NP == 10) ? 3 : NP == 12 ? 2 : emu_eb_staged(NP);
 }
 
-template <int NP, bool STAGE, bool DOT, bool SMALL>
+template <int NP, bool STAGE, bool DOT, EmuForm FORM>
 struct EmuCfg {
-  static constexpr int NP2 = NP * NP, NP3 = NP2 * NP, EB = emu_eb(NP, STAGE || SMALL), NT = NP2 * EB;
+  static constexpr int NP2 = NP * NP, NP3 = NP2 * NP, EB = emu_eb(NP, STAGE ? EMU_SMALL : FORM), NT = NP2 * EB;
   static constexpr int RS = NP | 1, PS = NP * RS, BUF = NP * PS;
   static constexpr int GS = (12 * NP3 + 3) / 4 * 4;  // factor block of one element (floats)
   // byte offsets: [factor block (TMA, offset 0)] [value buffers] [reduction slots, mbarrier]
@@ -337,9 +342,9 @@ __host__ __device__ constexpr bool emu_stage_fits(int NP) {
 
 // Blocks per SM the register allocation is held to; 0 = no floor (an explicit 1 lets the compiler
 // take far more registers).  Measured for the packed forms over floors of 0..7.
-__host__ __device__ constexpr int emu_min_blocks(int NP, bool stage, bool dot, bool small) {
-  if (small) return 0;
-  if (stage) return NP == 10 ? 4 : NP == 11 ? 3 : NP >= 12 ? 2 : 0;
+__host__ __device__ constexpr int emu_min_blocks(int NP, bool stage, bool dot, EmuForm form) {
+  if (form == EMU_SMALL) return 0;
+  if (stage || form == EMU_SCALAR) return NP == 10 ? 4 : NP == 11 ? 3 : NP >= 12 ? 2 : 0;
   if (dot) return NP == 4 ? 7 : NP == 10 || NP >= 12 ? 2 : 0;
   return NP == 4 ? 7 : NP == 6 || NP == 7 ? 4 : NP == 8 ? 5 : NP == 9 || NP == 11 ? 3 : NP >= 10 ? 2 : 0;
 }
@@ -351,7 +356,8 @@ __host__ __device__ constexpr int emu_min_blocks(int NP, bool stage, bool dot, b
 // Packed forms, GDOF/s at 1.6e7 nodes, modes 0 / 2 / 3: N = 3 61 / 59 / 55, 5 48 / 47 / 45, 6 41 / 43 /
 // 40, 7 41.5 / 44.5 / 40, 8 34.5 / 36.5 / 35, 9 31.6 / 31.0 / 30.8, 11 23.5 / 24.6 / 23.7, 12 23.5 / 19 /
 // 19, 13 16 / 17 / 20; mode 3 also leads at N = 14 and 15 (20.5 and 21.3 as chosen here).
-__host__ __device__ constexpr int emu_loop_mode(int NP) {
+__host__ __device__ constexpr int emu_loop_mode(int NP, EmuForm form) {
+  if (form == EMU_SCALAR) return NP == 7 || NP == 10 ? 0 : 2;
   return NP >= 14 ? 3 : (NP == 7 || NP == 8 || NP == 9 || NP == 11 || NP == 12) ? 2 : 0;
 }
 
@@ -359,12 +365,12 @@ __host__ __device__ constexpr int emu_loop_mode(int NP) {
 // two blocks per SM leave the loads exposed: N = 13 16.9 -> 19.9 GDOF/s, 15 +8%; slower below)
 __host__ __device__ constexpr bool emu_prefetch(int NP) { return NP >= 14; }
 
-template <int NP, bool BOXM, bool STAGE, bool DOT, bool SMALL>
-__global__ void __launch_bounds__(EmuCfg<NP, STAGE, DOT, SMALL>::NT, emu_min_blocks(NP, STAGE, DOT, SMALL)) k_apply_emu(const EmuParams<NP> P) {
-  using C = EmuCfg<NP, STAGE, DOT, SMALL>;
+template <int NP, bool BOXM, bool STAGE, bool DOT, EmuForm FORM>
+__global__ void __launch_bounds__(EmuCfg<NP, STAGE, DOT, FORM>::NT, emu_min_blocks(NP, STAGE, DOT, FORM)) k_apply_emu(const EmuParams<NP> P) {
+  using C = EmuCfg<NP, STAGE, DOT, FORM>;
   constexpr int N = NP - 1, NP2 = C::NP2, NP3 = C::NP3, EB = C::EB, NT = C::NT, RS = C::RS, PS = C::PS,
                 BUF = C::BUF, GS = C::GS;
-  constexpr bool PK = emu_packed(NP, DOT);
+  constexpr bool PK = emu_packed(NP, DOT, FORM);
   extern __shared__ __align__(128) unsigned char smem_raw[];
   static_assert(C::BUF_OFF % 16 == 0 && C::RED_OFF % 16 == 0, "shared-memory alignment");
   float *sG = reinterpret_cast<float *>(smem_raw);  // TMA destination: 16-byte aligned at offset 0
@@ -468,7 +474,7 @@ __global__ void __launch_bounds__(EmuCfg<NP, STAGE, DOT, SMALL>::NT, emu_min_blo
 
   // ---- phase 1: gradients ----
   float2 wt[NP];
-  if constexpr (emu_loop_mode(NP) == 3) {
+  if constexpr (emu_loop_mode(NP, FORM) == 3) {
     // direction 0: the r-line (j = a, k = b) into sr, 1: the s-line (i = a, k = b) into ss, 2: the
     // t-line (the column) into registers; the same base and stride address input and output
 #pragma unroll 1
@@ -488,7 +494,7 @@ __global__ void __launch_bounds__(EmuCfg<NP, STAGE, DOT, SMALL>::NT, emu_min_blo
         for (int i = 0; i < NP; ++i) dst[ib + i * is] = out[i];
       }
     }
-  } else if constexpr (emu_loop_mode(NP) == 2) {
+  } else if constexpr (emu_loop_mode(NP, FORM) == 2) {
     // the t-line (the column, in registers) inlined; the r-line (j = a, k = b) into sr and the
     // s-line (i = a, k = b) into ss through one loop body (the same base and stride address input
     // and output)
@@ -591,7 +597,7 @@ __global__ void __launch_bounds__(EmuCfg<NP, STAGE, DOT, SMALL>::NT, emu_min_blo
     wt[k] = dnorm(s, c);
   }
   float2 yt[NP];
-  if constexpr (emu_loop_mode(NP) == 3) {
+  if constexpr (emu_loop_mode(NP, FORM) == 3) {
     __syncthreads();
     // ---- phase 3: transposed contractions: 0 the r-line of sr, 1 the s-line of ss (in place),
     // 2 the column w_t in registers ----
@@ -612,7 +618,7 @@ __global__ void __launch_bounds__(EmuCfg<NP, STAGE, DOT, SMALL>::NT, emu_min_blo
         for (int i = 0; i < NP; ++i) buf[ib + i * is] = out[i];
       }
     }
-  } else if constexpr (emu_loop_mode(NP) == 2) {
+  } else if constexpr (emu_loop_mode(NP, FORM) == 2) {
     df_line<NP, true, PK>(P, wt, yt);  // D^T w_t of the column
     __syncthreads();
     // ---- phase 3: transposed contractions: 0 the r-line of sr, 1 the s-line of ss (in place) ----
@@ -717,33 +723,65 @@ __global__ void __launch_bounds__(EmuCfg<NP, STAGE, DOT, SMALL>::NT, emu_min_blo
   }
 }
 
-template <int NP, bool BOXM, bool STAGE, bool DOT, bool SMALL>
+template <int NP, bool BOXM, bool STAGE, bool DOT, EmuForm FORM>
 sem_status launch_k(const EmuParams<NP> &p, cudaStream_t s) {
-  using C = EmuCfg<NP, STAGE, DOT, SMALL>;
+  using C = EmuCfg<NP, STAGE, DOT, FORM>;
   const unsigned grid = (unsigned)((p.E + C::EB - 1) / C::EB);
   if (p.partials && grid > SEM_MAX_PARTIALS) return sem_fail(SEM_ERR_INVALID, "too many elements for fused dot");
   static std::atomic<unsigned long long> attr_done;
-  const cudaError_t e = set_smem_limit_once(k_apply_emu<NP, BOXM, STAGE, DOT, SMALL>, C::SMEM, attr_done);
+  const cudaError_t e = set_smem_limit_once(k_apply_emu<NP, BOXM, STAGE, DOT, FORM>, C::SMEM, attr_done);
   if (e != cudaSuccess) return sem_fail(SEM_ERR_CUDA, std::string("emu attributes: ") + cudaGetErrorString(e));
   if constexpr (DOT)
-    SEM_CUDA_TRY(launch_dependent(k_apply_emu<NP, BOXM, STAGE, DOT, SMALL>, grid, C::NT, C::SMEM, s, p));
+    SEM_CUDA_TRY(launch_dependent(k_apply_emu<NP, BOXM, STAGE, DOT, FORM>, grid, C::NT, C::SMEM, s, p));
   else
-    k_apply_emu<NP, BOXM, STAGE, DOT, SMALL><<<grid, C::NT, C::SMEM, s>>>(p);
+    k_apply_emu<NP, BOXM, STAGE, DOT, FORM><<<grid, C::NT, C::SMEM, s>>>(p);
   return SEM_OK;
 }
 
-template <int NP, bool STAGE, bool SMALL>
-sem_status launch_b(const EmuParams<NP> &p, bool boxm, bool dot, cudaStream_t s) {
-  if (dot) return boxm ? launch_k<NP, true, STAGE, true, SMALL>(p, s) : launch_k<NP, false, STAGE, true, SMALL>(p, s);
-  return boxm ? launch_k<NP, true, STAGE, false, SMALL>(p, s) : launch_k<NP, false, STAGE, false, SMALL>(p, s);
+// Which form a problem of E elements takes.  The fuller blocks of EMU_FULL (and their register floors, which
+// spill) serve a chip full of blocks; a few blocks, or a last wave that is nearly empty, want smaller ones and
+// a short chain of instructions per thread.  The limits are elements per SM; plain applies, us, full / small /
+// scalar (caches warm):
+//   N = 6   128 elements 13.5 / 10.7 / 11.0, 1200 18.1 / 15.5 / 15.2, 1728 22.8 / 23.3 / 20.0, 2160 23.1 / 26.5 / 28.0
+//   N = 7   288 9.9 / 10.8 / 11.3, 729 14.7 / 14.2 / 13.9, 1200 17.9 / 20.8 / 17.3, 1573 24.0 / 25.4 / 26.4
+//   N = 8   128 17.2 / 12.7 / 12.2, 576 23.7 / 17.4 / 15.9, 729 24.0 / 24.8 / 20.0, 891 24.2 / 26.7 / 27.0
+//   N = 9   128 21.9 / 12.0 / 15.0, 441 22.7 / 19.8 / 18.8, 729 32.4 / 31.4 / 35.8, 1200 49.4 / 48.9 / 51.8 (1000:
+//           47.2 full, 42.7 scalar; two blocks of the scalar form fill an SM four at a time)
+//   N = 11  128 31.0 / 16.4 / 20.0, 288 31.6 / 30.3 / 26.8, 576 47.9 / 57.6 / 49.8, 891 78.0 / 91.5 / 76.0
+// The kernel of a CG step has its own order (an iteration, us): N = 6 729 elements 30.0 / 31.7 / 33.1, N = 8 27
+// elements 30.9 / 29.8 / 29.9, 729 43.5 / 44.1 / 44.0, N = 9 1000 85.7 / 74.3 / 78.2, 2535 154.6 / 151.4 / 165.6, N = 11
+// 441 74.8 / 74.5 / 79.1, 1000 137 / 165 / 157.
+__host__ __device__ constexpr bool emu_has(int NP, EmuForm form, bool dot) {
+  return form == EMU_FULL || (form == EMU_SMALL ? NP == 10 || NP == 12
+                                                : NP == 9 || (!dot && (NP == 7 || NP == 8 || NP == 10 || NP == 12)));
+}
+inline EmuForm emu_form(int NP, int64_t E, bool dot) {
+  const int64_t S = SEM_SMS;
+  switch (NP) {
+    case 7: return !dot && E <= 13 * S ? EMU_SCALAR : EMU_FULL;
+    case 8: return !dot && E > 3 * S && E <= 8 * S ? EMU_SCALAR : EMU_FULL;
+    case 9: return E <= 5 * S ? EMU_SCALAR : EMU_FULL;
+    case 10:
+      if (E > (dot ? 20 : 8) * S) return EMU_FULL;
+      return !dot && (E - 1) / (2 * S) % 2 == 1 ? EMU_SCALAR : EMU_SMALL;
+    case 12:
+      if (E > (dot ? 4 : 6) * S) return EMU_FULL;
+      return !dot && E > S ? EMU_SCALAR : EMU_SMALL;
+    default: return EMU_FULL;
+  }
 }
 
-// Whether a problem is too small for the fuller blocks of emu_eb: these (and their register floors, which
-// spill) serve a chip full of blocks; below two blocks per SM a thread's own latency counts.
-// 27 elements at N = 9 / 11, us: fuller blocks 21.4 / 29.9, smaller 10.6 / 16.0 (with one element per
-// block and the floors: 13.4 / 19.4).
-__host__ __device__ constexpr bool emu_has_small(int NP) { return emu_eb(NP, false) != emu_eb(NP, true); }
-inline bool emu_small(int NP, int64_t E) { return emu_has_small(NP) && E < (int64_t)2 * 152 * emu_eb(NP, false); }
+template <int NP, bool STAGE, EmuForm FORM>
+sem_status launch_b(const EmuParams<NP> &p, bool boxm, bool dot, cudaStream_t s) {
+  if (dot) {
+    if constexpr (emu_has(NP, FORM, true))
+      return boxm ? launch_k<NP, true, STAGE, true, FORM>(p, s) : launch_k<NP, false, STAGE, true, FORM>(p, s);
+  } else {
+    if constexpr (emu_has(NP, FORM, false))
+      return boxm ? launch_k<NP, true, STAGE, false, FORM>(p, s) : launch_k<NP, false, STAGE, false, FORM>(p, s);
+  }
+  return sem_fail(SEM_ERR_INVALID, "emu apply: form not built");  // emu_form asks for no such form
+}
 
 template <int NP>
 sem_status launch_emu(const sem_handle *h, const double *u, double *y, double *partials, SemScalars *scal,
@@ -791,12 +829,16 @@ sem_status launch_emu(const sem_handle *h, const double *u, double *y, double *p
   if (partials && !scal) return sem_fail(SEM_ERR_INVALID, "fused dot needs the solver scalars");
   const bool boxm = p.glo == nullptr && p.bc != SEM_BC_MASK;
   // variant 0: factor block staged by TMA when it fits; other variants read factors directly, and so
-  // does the automatic choice (-1) except on small problems at N = 5 (64 elements: 7.1 against 8.8 us)
-  const bool small = emu_small(NP, p.E);
-  const bool stage = emu_stage_fits(NP) && (h->apply_variant == 0 || (h->apply_variant < 0 && NP == 6 && small));
-  const sem_status st = stage ? launch_b<NP, emu_stage_fits(NP), false>(p, boxm, partials != nullptr, s)
-                        : small ? launch_b<NP, false, emu_has_small(NP)>(p, boxm, partials != nullptr, s)
-                                             : launch_b<NP, false, false>(p, boxm, partials != nullptr, s);
+  // does the automatic choice (-1) except on small problems at N = 5 (64 elements: 7.1 against 8.8 us; 2535
+  // elements: plain 17.4 against 19.4 us, the kernel of a CG step 43.2 against 40.0)
+  const bool dot = partials != nullptr;
+  const bool stage = emu_stage_fits(NP) && (h->apply_variant == 0 || (h->apply_variant < 0 && NP == 6 &&
+                                                                      p.E < (dot ? 14 : 28) * (int64_t)SEM_SMS));
+  const EmuForm form = emu_form(NP, p.E, dot);
+  const sem_status st = stage                ? launch_b<NP, emu_stage_fits(NP), EMU_FULL>(p, boxm, dot, s)
+                        : form == EMU_SCALAR ? launch_b<NP, false, EMU_SCALAR>(p, boxm, dot, s)
+                        : form == EMU_SMALL  ? launch_b<NP, false, EMU_SMALL>(p, boxm, dot, s)
+                                             : launch_b<NP, false, EMU_FULL>(p, boxm, dot, s);
   if (st != SEM_OK) return st;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return sem_fail(SEM_ERR_CUDA, std::string("emu apply launch: ") + cudaGetErrorString(e));

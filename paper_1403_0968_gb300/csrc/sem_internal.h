@@ -30,6 +30,9 @@ struct NvtxRange {
 
 // Number of partial-sum slots a solver reduction may use, and groups of 256 of them.
 #define SEM_MAX_PARTIALS (1 << 20)
+// SMs of a GB300.  The limits of the size rules were measured there; another count shifts the choice between
+// forms of a kernel, not their results.
+#define SEM_SMS 152
 #define SEM_MAX_GROUPS (SEM_MAX_PARTIALS / 256)
 
 // Device-resident solver scalars.  Every CG scalar lives here so that no iteration needs the
