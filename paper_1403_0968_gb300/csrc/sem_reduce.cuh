@@ -90,6 +90,8 @@ __device__ __forceinline__ bool warp_publish_2level(double v, double *partials, 
     __threadfence();
     last = atomicAdd(&gtickets[group], 1u) == gsize - 1u;
   }
+  // a shuffle alone does not order the lanes' memory accesses: the other lanes' loads come after lane 0's ticket
+  __syncwarp();
   if (!__shfl_sync(0xffffffffu, last, 0)) return false;
   __threadfence();
   const double gsum = warp_sum_partials(partials + group * 256u, (int)gsize);
@@ -99,6 +101,7 @@ __device__ __forceinline__ bool warp_publish_2level(double v, double *partials, 
     __threadfence();
     last = atomicAdd(ticket, 1u) == ngroups - 1u;
   }
+  __syncwarp();
   if (!__shfl_sync(0xffffffffu, last, 0)) return false;
   __threadfence();
   *total = warp_sum_partials(gpartials, (int)ngroups);
