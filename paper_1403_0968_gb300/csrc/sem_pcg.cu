@@ -18,6 +18,7 @@
 #include <algorithm>
 #include <string>
 
+#include "sem_graph.h"
 #include "sem_internal.h"
 #include "sem_reduce.cuh"
 
@@ -390,30 +391,6 @@ struct History {
   }
 };
 
-// Captures what `body` launches and makes it an executable graph (*exec).  The legacy default stream
-// cannot be captured: its work is captured on a stream of its own and replayed on the default one.
-template <typename F>
-sem_status capture_graph(cudaStream_t st, cudaGraphExec_t *exec, F body) {
-  cudaStream_t cap = st;
-  if (!st) SEM_CUDA_TRY(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
-  cudaGraph_t g = nullptr;
-  sem_status s = SEM_OK;
-  cudaError_t ce = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
-  if (ce == cudaSuccess) {
-    s = body(cap);
-    ce = cudaStreamEndCapture(cap, &g);
-  }
-  if (!st) cudaStreamDestroy(cap);
-  if (s == SEM_OK && ce != cudaSuccess)
-    s = sem_fail(SEM_ERR_CUDA, std::string("graph capture: ") + cudaGetErrorString(ce));
-  if (s == SEM_OK) {
-    ce = cudaGraphInstantiate(exec, g, 0);
-    if (ce != cudaSuccess) s = sem_fail(SEM_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(ce));
-  }
-  if (g) cudaGraphDestroy(g);
-  return s;
-}
-
 // One block of `count` CG iterations on type T.
 template <typename T>
 sem_status cg_block(sem_handle *h, int prec, int count, T *x, T *p, T *r, T *Ap, const T *dinv, cudaStream_t st) {
@@ -433,12 +410,11 @@ sem_status cg_block(sem_handle *h, int prec, int count, T *x, T *p, T *r, T *Ap,
 }
 
 // Runs CG from the state set up by k_cg_init until convergence, breakdown or max_it.
-// exec: the graph of check_every iterations, captured at its first use and kept by the caller for its
-// later calls with the same vectors.  hist (may be null) gets (it0 + iterations, sqrt(rr / bb)) at
+// graph: that of check_every iterations, kept by the caller for its later calls with the same vectors.  hist (may be null) gets (it0 + iterations, sqrt(rr / bb)) at
 // each host check.
 template <typename T>
 sem_status cg_run(sem_handle *h, int prec, const sem_pcg_opts *o, T *x, T *p, T *r, T *Ap, const T *dinv,
-                  cudaStream_t st, cudaGraphExec_t *exec, int *iters, double *rr_out, int budget,
+                  cudaStream_t st, StepGraph *graph, int *iters, double *rr_out, int budget,
                   History *hist = nullptr, int it0 = 0, double bb = 0.0) {
   SemScalars hs;
   sem_status s = read_scalars(h, &hs, st);
@@ -447,21 +423,9 @@ sem_status cg_run(sem_handle *h, int prec, const sem_pcg_opts *o, T *x, T *p, T 
   const int every = std::max(1, o->check_every);
   while (!hs.converged && !hs.breakdown && hs.iter < budget) {
     const int count = std::min(every, budget - hs.iter);
-    if (o->use_graph && count == every) {
-      if (!*exec) {
-        s = capture_graph(st, exec,
-                          [&](cudaStream_t cap) { return cg_block<T>(h, prec, count, x, p, r, Ap, dinv, cap); });
-        if (s != SEM_OK) break;
-      }
-      const cudaError_t ce = cudaGraphLaunch(*exec, st);
-      if (ce != cudaSuccess) {
-        s = sem_fail(SEM_ERR_CUDA, std::string("graph launch: ") + cudaGetErrorString(ce));
-        break;
-      }
-    } else {
-      s = cg_block<T>(h, prec, count, x, p, r, Ap, dinv, st);
-      if (s != SEM_OK) break;
-    }
+    auto block = [&](cudaStream_t on) { return cg_block<T>(h, prec, count, x, p, r, Ap, dinv, on); };
+    s = o->use_graph && count == every ? replay(st, graph, block) : block(st);
+    if (s != SEM_OK) break;
     s = read_scalars(h, &hs, st);
     if (s != SEM_OK) break;
     if (hist && bb > 0) hist->add(it0 + hs.iter, sqrt(hs.rr / bb));
@@ -523,12 +487,7 @@ extern "C" sem_status sem_pcg(sem_handle *h, const double *d_b, double *d_x, con
   const int64_t G = h->G;
   sem_status s = SEM_OK;
   SemScalars hs;
-  struct Exec {  // the solve's step graph, released on every way out
-    cudaGraphExec_t e = nullptr;
-    ~Exec() {
-      if (e) cudaGraphExecDestroy(e);
-    }
-  } exec;
+  StepGraph steps;  // released on every way out
   SEM_CUDA_TRY(cudaMemsetAsync(h->scal, 0, sizeof(SemScalars), st));
 
   if (o->mode == SEM_SOLVE_FP64) {
@@ -550,7 +509,7 @@ extern "C" sem_status sem_pcg(sem_handle *h, const double *d_b, double *d_x, con
       const double bb = hs.bb;
       int iters = 0;
       double rr = 0.0;
-      s = cg_run<double>(h, prec64, o, d_x, h->p64, h->r64, h->Ap64, h->dinv64, st, &exec.e, &iters, &rr,
+      s = cg_run<double>(h, prec64, o, d_x, h->p64, h->r64, h->Ap64, h->dinv64, st, &steps, &iters, &rr,
                          std::max(1, o->max_it - total), &hist, total, bb);
       total += iters;
       res->recursive_relres = bb > 0 ? sqrt(rr / bb) : 0.0;
@@ -606,7 +565,7 @@ extern "C" sem_status sem_pcg(sem_handle *h, const double *d_b, double *d_x, con
                                                 h->dinv32, h->scal, h->partials, inner * inner);
       int iters = 0;
       double rr = 0.0;
-      s = cg_run<float>(h, inner_prec, o, h->x32, h->p32, h->r32, h->Ap32, h->dinv32, st, &exec.e, &iters, &rr,
+      s = cg_run<float>(h, inner_prec, o, h->x32, h->p32, h->r32, h->Ap32, h->dinv32, st, &steps, &iters, &rr,
                         std::max(1, o->max_it - total));
       total += iters;
       if (s == SEM_ERR_NOCONV) s = SEM_OK;  // a partial inner solve still improves x
@@ -647,12 +606,7 @@ extern "C" sem_status sem_pcg(sem_handle *h, const double *d_b, double *d_x, con
       while (s == SEM_OK && !hs.converged && !hs.breakdown && hs.iter < o->max_it) {
         const int count = std::min(every, o->max_it - hs.iter);
         if (graph && eager_done && count == every) {
-          if (!exec.e) {
-            s = capture_graph(st, &exec.e, [&](cudaStream_t cap) { return fcg_block(h, prec64, count, d_x, cap); });
-            if (s != SEM_OK) break;
-          }
-          const cudaError_t ce = cudaGraphLaunch(exec.e, st);
-          if (ce != cudaSuccess) s = sem_fail(SEM_ERR_CUDA, std::string("graph launch: ") + cudaGetErrorString(ce));
+          s = replay(st, &steps, [&](cudaStream_t on) { return fcg_block(h, prec64, count, d_x, on); });
         } else {
           s = fcg_block(h, prec64, graph && !eager_done ? 1 : count, d_x, st);
           eager_done = true;
