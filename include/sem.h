@@ -370,7 +370,7 @@ sem_status sem_batch_set_fused(sem_batch *b, int32_t fused);
 sem_status sem_batch_get_fused(const sem_batch *b, int32_t *available, int32_t *in_use);
 
 /* Polls after which a grid-wide wait of the fused step kernel gives up (polls < 0: the default,
-   2^22 polls of about 64 ns or more; 0: every wait but the last block's gives up at once).  A step whose
+   2^22 polls of about 256 ns; 0: every wait but the last block's gives up at once).  A step whose
    wait gave up leaves its blocks without finishing the step and sem_batch_pcg returns
    SEM_ERR_TIMEOUT (the flag and the barrier are cleared for later solves): this is how the
    timeout path is tested, with no fault and no hang.  Errors: SEM_ERR_INVALID. */

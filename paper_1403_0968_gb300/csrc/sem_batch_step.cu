@@ -274,7 +274,8 @@ __device__ __forceinline__ bool grid_barrier(const FusedParams &P) {
       atomicAdd(P.bar + 1, 1u);
     } else {
       ok = 0;
-      for (uint32_t t = 0; t < P.wait_polls; ++t) {
+      // a poll is four looks, 64 ns apart: a block goes on sooner, the limit stays about 256 ns a poll
+      for (uint64_t t = 0; t < (uint64_t)P.wait_polls * 4; ++t) {
         if (*gen != g) {
           ok = 1;
           break;
