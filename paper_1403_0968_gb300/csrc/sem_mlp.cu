@@ -405,8 +405,8 @@ extern "C" sem_status sem_mlp_train_scratch(int32_t N, int32_t h1, int32_t h2, i
   if (s != SEM_OK) return s;
   if (batch < 1 || !bytes) return sem_fail(SEM_ERR_INVALID, "bad batch");
   const int n = N + 1, n3 = n * n * n;
-  // H1, H2, O, dO, dH2, dH1 activations + gradient + loss
-  *bytes = ((size_t)batch * (2 * h1 + 2 * h2 + 2 * n3) + (size_t)P) * 4 + 64;
+  // activations H1, H2 and the gradients dO, dH2, dH1
+  *bytes = (size_t)batch * (2 * h1 + 2 * h2 + n3) * 4 + 64;
   return SEM_OK;
 }
 
@@ -467,8 +467,8 @@ extern "C" sem_status sem_mlp_train_step(int32_t N, int32_t h1, int32_t h2, floa
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int n = N + 1;
   const Shape S = shape_of(n * n * n, h1, h2);
-  float *H1 = static_cast<float *>(d_scratch), *H2 = H1 + (size_t)batch * h1, *O = H2 + (size_t)batch * h2;
-  float *dO = O + (size_t)batch * S.nout, *dH2 = dO + (size_t)batch * S.nout, *dH1 = dH2 + (size_t)batch * h2;
+  float *H1 = static_cast<float *>(d_scratch), *H2 = H1 + (size_t)batch * h1, *dO = H2 + (size_t)batch * h2;
+  float *dH2 = dO + (size_t)batch * S.nout, *dH1 = dH2 + (size_t)batch * h2;
   float *W = d_params;
   using namespace mlpg;
   // gradient of the weights at oW and the bias at ob, and their update
