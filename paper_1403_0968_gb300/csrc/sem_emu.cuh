@@ -744,10 +744,11 @@ sem_status launch_k(const EmuParams<NP> &p, cudaStream_t s) {
 // scalar (caches warm):
 //   N = 6   128 elements 13.5 / 10.7 / 11.0, 1200 18.1 / 15.5 / 15.2, 1728 22.8 / 23.3 / 20.0, 2160 23.1 / 26.5 / 28.0
 //   N = 7   288 9.9 / 10.8 / 11.3, 729 14.7 / 14.2 / 13.9, 1200 17.9 / 20.8 / 17.3, 1573 24.0 / 25.4 / 26.4
-//   N = 8   128 17.2 / 12.7 / 12.2, 576 23.7 / 17.4 / 15.9, 729 24.0 / 24.8 / 20.0, 891 24.2 / 26.7 / 27.0
+//   N = 8   128 17.2 / 12.7 / 12.2, 576 23.7 / 17.4 / 15.9, 729 24.0 / 24.8 / 20.0, 891 24.2 / 26.7 / 27.0, 972 31.0 full
 //   N = 9   128 21.9 / 12.0 / 15.0, 441 22.7 / 19.8 / 18.8, 729 32.4 / 31.4 / 35.8, 1200 49.4 / 48.9 / 51.8 (1000:
 //           47.2 full, 42.7 scalar; two blocks of the scalar form fill an SM four at a time)
-//   N = 11  128 31.0 / 16.4 / 20.0, 288 31.6 / 30.3 / 26.8, 576 47.9 / 57.6 / 49.8, 891 78.0 / 91.5 / 76.0
+//   N = 11  128 31.0 / 16.4 / 20.0, 288 31.6 / 30.3 / 26.8, 441 44.7 / 44.1 / 42.3 (caches cold 54 / 58 / 64), 576 47.9 /
+//           57.6 / 49.8, 729 74.5 / 71.9 / 66.5, 891 78.0 / 91.5 / 76.0
 // The kernel of a CG step has its own order (an iteration, us): N = 6 729 elements 30.0 / 31.7 / 33.1, N = 8 27
 // elements 30.9 / 29.8 / 29.9, 729 43.5 / 44.1 / 44.0, N = 9 1000 85.7 / 74.3 / 78.2, 2535 154.6 / 151.4 / 165.6, N = 11
 // 441 74.8 / 74.5 / 79.1, 1000 137 / 165 / 157.
@@ -760,12 +761,12 @@ inline EmuForm emu_form(int NP, int64_t E, bool dot) {
   switch (NP) {
     case 7: return !dot && E <= 13 * S ? EMU_SCALAR : EMU_FULL;
     case 8: return !dot && E > 3 * S && E <= 8 * S ? EMU_SCALAR : EMU_FULL;
-    case 9: return E <= 5 * S ? EMU_SCALAR : EMU_FULL;
+    case 9: return E <= 5 * S || (E > 6 * S && E <= 8 * S) ? EMU_SCALAR : EMU_FULL;  // two full blocks per SM between
     case 10:
       if (E > (dot ? 20 : 8) * S) return EMU_FULL;
       return !dot && (E - 1) / (2 * S) % 2 == 1 ? EMU_SCALAR : EMU_SMALL;
     case 12:
-      if (E > (dot ? 4 : 6) * S) return EMU_FULL;
+      if (E > (dot ? 4 : 6) * S || (!dot && E > 2 * S && E <= 4 * S)) return EMU_FULL;
       return !dot && E > S ? EMU_SCALAR : EMU_SMALL;
     default: return EMU_FULL;
   }

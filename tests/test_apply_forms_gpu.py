@@ -9,14 +9,14 @@ import workloads as W
 pytestmark = pytest.mark.gpu
 TOL = 1e-12  # of max |y|: the bound of every FP64-accurate apply
 
-# double-float: N = 5 staged below 4256 elements; 6 scalar to 1976, then blocks of 5; 7 scalar from 457 to 1216;
-# 8 scalar to 760, then blocks of 3; 9 small to 304 and from 609 to 912, scalar between and to 1216, then blocks
-# of 3; 11 small to 152, scalar to 912, then blocks of 2
-EMU = [(5, (7, 16, 38)), (5, (16, 16, 17)), (5, (5, 23, 37)), (5, (12, 13, 13)), (6, (8, 13, 19)), (6, (12, 13, 13)), (6, (1, 1, 1)),
-       (7, (3, 8, 19)), (7, (8, 8, 8)), (7, (8, 8, 19)), (7, (11, 11, 11)), (8, (4, 10, 19)), (8, (9, 9, 10)),
-       (8, (10, 10, 10)), (9, (1, 16, 19)), (9, (7, 7, 7)), (9, (2, 16, 19)), (9, (8, 9, 9)), (9, (4, 16, 16)),
-       (9, (4, 16, 19)), (9, (11, 11, 11)), (11, (1, 8, 19)), (11, (4, 6, 7)), (11, (3, 16, 19)), (11, (10, 10, 10)),
-       (11, (9, 11, 11))]
+# double-float: N = 5 staged below 4256 elements; 6 scalar to 1976, then blocks of 5; 7 scalar from 457 to 1216; 8 scalar
+# to 760 and from 913 to 1216, else blocks of 3; 9 small to 304 and from 609 to 912, scalar between and to 1216, then
+# blocks of 3; 11 small to 152, scalar to 304 and from 609 to 912, else blocks of 2
+EMU = [(5, (7, 16, 38)), (5, (16, 16, 17)), (5, (5, 23, 37)), (5, (12, 13, 13)), (6, (1, 1, 1)), (6, (8, 13, 19)),
+       (6, (12, 13, 13)), (7, (3, 8, 19)), (7, (8, 8, 8)), (7, (8, 8, 19)), (7, (11, 11, 11)), (8, (4, 10, 19)),
+       (8, (9, 9, 10)), (8, (10, 10, 10)), (8, (11, 11, 11)), (9, (1, 16, 19)), (9, (7, 7, 7)), (9, (2, 16, 19)),
+       (9, (8, 9, 9)), (9, (4, 16, 16)), (9, (4, 16, 19)), (9, (11, 11, 11)), (11, (1, 8, 19)), (11, (4, 6, 7)),
+       (11, (7, 7, 9)), (11, (3, 16, 19)), (11, (10, 10, 10)), (11, (9, 11, 11))]
 COLS = [(14, (4, 4, 19)), (14, (7, 7, 7)), (13, (5, 7, 9)), (6, (2, 2, 2)), (12, (2, 2, 2))]
 
 
