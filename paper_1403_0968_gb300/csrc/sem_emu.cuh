@@ -240,14 +240,14 @@ enum EmuForm { EMU_FULL, EMU_SMALL, EMU_SCALAR };
 
 // Whether an order runs its line products and factor scaling in packed form (DOT: with the fused
 // reduction of a CG step, whose registers come on top).  Measured, GDOF/s at 1.6e7 nodes, scalar /
-// packed: plain N = 2 59 / 57, 4 52 / 51, 10 32 / 30, 7 42 / 44.5, 11 20.6 / 24.6, 15 17 / 26; DOT
+// packed: plain N = 2 59 / 57, 4 52 / 51, 10 32 / 30, 7 42 / 44.5, 11 20.6 / 24.6, 15 17 / 21; DOT
 // N = 5 43 / 37, 6 36 / 36, 7 42 / 40, 8 35.5 / 28, 9 27 / 30, 15 14.5 / 21.
 __host__ __device__ constexpr bool emu_packed(int NP, bool dot, EmuForm form) {
   if (form == EMU_SCALAR) return false;
   return NP == 4 || NP == 10 || NP >= 12 || (!dot && NP >= 6 && NP <= 9);
 }
-// whether the even and odd parts of a line are formed together too (N = 15 one after the other: 26 GDOF/s
-// against 22 in the build the form was chosen in, where its 128 registers did not hold both; 21.3 now)
+// whether the even and odd parts of a line are formed together too (N = 15, whose 128 registers do not hold
+// both, one after the other: 20% faster in the build the choice was made in)
 __host__ __device__ constexpr bool emu_packed_parts(int NP) { return NP <= 14; }
 
 // out = M v for one line, M = D (TRANS false) or D^T (TRANS true), in double-float: the odd part
@@ -749,25 +749,28 @@ sem_status launch_k(const EmuParams<NP> &p, cudaStream_t s) {
 //           47.2 full, 42.7 scalar; two blocks of the scalar form fill an SM four at a time)
 //   N = 11  128 31.0 / 16.4 / 20.0, 288 31.6 / 30.3 / 26.8, 441 44.7 / 44.1 / 42.3 (caches cold 54 / 58 / 64), 576 47.9 /
 //           57.6 / 49.8, 729 74.5 / 71.9 / 66.5, 891 78.0 / 91.5 / 76.0
-// The kernel of a CG step has its own order (an iteration, us): N = 6 729 elements 30.0 / 31.7 / 33.1, N = 8 27
-// elements 30.9 / 29.8 / 29.9, 729 43.5 / 44.1 / 44.0, N = 9 1000 85.7 / 74.3 / 78.2, 2535 154.6 / 151.4 / 165.6, N = 11
-// 441 74.8 / 74.5 / 79.1, 1000 137 / 165 / 157.
+// The kernel of a CG step has its own order (an iteration, us): N = 6 27 elements 26.1 / 25.1 / 27.2, 1000 35.6 / 34.5 /
+// 35.3, N = 8 27 30.9 / 29.8 / 29.9, 729 43.5 / 44.1 / 44.0, 1000 53.4 / 55.7 / 55.7, N = 9 1000 85.7 / 74.3 / 78.2, 2535
+// 154.6 / 151.4 / 165.6 (explicit numbering, 2744: 240 full, 306 small), N = 11 200 55.2 / 53.4 / 46.9, 441 74.8 / 74.5 / 79.1,
+// 1000 137 / 165 / 157 (explicit numbering, 216: 80 small, 66 scalar; 729: 177 full, 162 scalar).
 __host__ __device__ constexpr bool emu_has(int NP, EmuForm form, bool dot) {
-  return form == EMU_FULL || (form == EMU_SMALL ? NP == 10 || NP == 12
-                                                : NP == 9 || (!dot && (NP == 7 || NP == 8 || NP == 10 || NP == 12)));
+  return form == EMU_FULL || (form == EMU_SMALL ? NP == 10 || NP == 12 || (dot && NP == 7)
+                                                : NP == 9 || NP == 12 || (!dot && (NP == 7 || NP == 8 || NP == 10)));
 }
-inline EmuForm emu_form(int NP, int64_t E, bool dot) {
+inline EmuForm emu_form(int NP, int64_t E, bool dot, bool boxm) {
   const int64_t S = SEM_SMS;
   switch (NP) {
-    case 7: return !dot && E <= 13 * S ? EMU_SCALAR : EMU_FULL;
+    case 7: return dot ? (E <= 10 * S ? EMU_SMALL : EMU_FULL) : E <= 13 * S ? EMU_SCALAR : EMU_FULL;
     case 8: return !dot && E > 3 * S && E <= 8 * S ? EMU_SCALAR : EMU_FULL;
-    case 9: return E <= 5 * S || (E > 6 * S && E <= 8 * S) ? EMU_SCALAR : EMU_FULL;  // two full blocks per SM between
+    case 9: return E <= 5 * S || (!dot && E > 6 * S && E <= 8 * S) ? EMU_SCALAR : EMU_FULL;
     case 10:
-      if (E > (dot ? 20 : 8) * S) return EMU_FULL;
+      if (E > (dot && boxm ? 20 : dot ? 6 : 8) * S) return EMU_FULL;
       return !dot && (E - 1) / (2 * S) % 2 == 1 ? EMU_SCALAR : EMU_SMALL;
     case 12:
-      if (E > (dot ? 4 : 6) * S || (!dot && E > 2 * S && E <= 4 * S)) return EMU_FULL;
-      return !dot && E > S ? EMU_SCALAR : EMU_SMALL;
+      if (E <= S) return EMU_SMALL;
+      if (E <= 2 * S || (dot && !boxm && E <= 6 * S)) return EMU_SCALAR;
+      if (E <= 4 * S) return dot ? EMU_SMALL : EMU_FULL;
+      return !dot && E <= 6 * S ? EMU_SCALAR : EMU_FULL;
     default: return EMU_FULL;
   }
 }
@@ -835,7 +838,7 @@ sem_status launch_emu(const sem_handle *h, const double *u, double *y, double *p
   const bool dot = partials != nullptr;
   const bool stage = emu_stage_fits(NP) && (h->apply_variant == 0 || (h->apply_variant < 0 && NP == 6 &&
                                                                       p.E < (dot ? 14 : 28) * (int64_t)SEM_SMS));
-  const EmuForm form = emu_form(NP, p.E, dot);
+  const EmuForm form = emu_form(NP, p.E, dot, boxm);
   const sem_status st = stage                ? launch_b<NP, emu_stage_fits(NP), EMU_FULL>(p, boxm, dot, s)
                         : form == EMU_SCALAR ? launch_b<NP, false, EMU_SCALAR>(p, boxm, dot, s)
                         : form == EMU_SMALL  ? launch_b<NP, false, EMU_SMALL>(p, boxm, dot, s)
