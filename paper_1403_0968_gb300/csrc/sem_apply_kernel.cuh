@@ -289,18 +289,22 @@ __host__ __device__ constexpr size_t apply_smem() {
 // Minimum resident blocks the FP32 kernel's registers are held to at high order, where one
 // element per block otherwise leaves one or two blocks per SM; 0 = no floor (an explicit 1 lets the
 // compiler take more registers).
-// Plain applies with explicit numbering take registers for the node ids.  Where the compiler gave an order fewer
-// blocks per SM for them than a box has, these are asked for: on the fly, us at about 7e6 nodes with the
-// floor / without: N = 5 142 / 160, 7 128 / 160, 9 166 / 197, 11 198 / 242; BF16 N = 11 149 / 168.
-template <typename T, typename TG, bool PLAIN_GLO>
+// Explicit numbering takes registers for the node ids.  Where the compiler would give an order fewer blocks per
+// SM for them than a box has, these are asked for.  Plain applies, on the fly, us at about 7e6 nodes with the floor /
+// without: N = 5 142 / 160, 7 128 / 160, 9 166 / 197, 11 198 / 242; BF16 N = 11 149 / 168.
+template <typename T, typename TG, bool BOXM, bool DOT>
 __host__ __device__ constexpr int apply_min_blocks(int NP, int EB) {
-  if (PLAIN_GLO && is_otf<TG>() && EB == apply_eb_default(NP)) {
-    if (NP == 5 || NP == 6) return 7;
-    if (NP == 10) return 6;
-    if (NP == 12) return 4;
+  if (!BOXM && is_otf<TG>()) {
+    if (EB == apply_eb_default(NP)) {
+      if (NP == 6 || (NP == 5 && !DOT)) return 7;
+      if (NP == 10 && !DOT) return 6;
+      if (NP == 12 && !DOT) return 4;
+    }
+    if (NP == 8 && EB == 1 && !DOT) return 14;
+  } else if (!BOXM && sizeof(T) == 4 && EB == 1) {
+    if (NP == 7 && DOT) return 20;
+    if (NP == 12) return DOT ? 5 : 6;
   }
-  if (PLAIN_GLO && is_otf<TG>() && NP == 8 && EB == 1) return 14;
-  if (PLAIN_GLO && sizeof(T) == 4 && NP == 12 && EB == 1) return 6;
   return (sizeof(T) == 4 && EB == 1 && NP >= 13 && NP <= 15) ? 2 : 0;  // measured: +15-35% at N = 12..14
 }
 
@@ -335,18 +339,18 @@ __host__ __device__ constexpr bool apply_packed(int NP) {
 // TG: storage type of the factors (T, or BF16 with T = float: half the factor traffic).
 // DOT: with the sum of a CG step, run when P.partials is set.  Explicit numbering has plain applies without that
 // code, with scalar line products and without held factors (PREF): on top of its node ids the registers of
-// any of the three cost more than they gave.  Explicit numbering at about 7e6 nodes, us, with all three / without:
+// any of the three cost more than they gave (not in a CG step's kernel).  Explicit numbering at about 7e6 nodes, us, with all three / without:
 // FP32 N = 4 129 / 95, 5 158 / 118, 9 174 / 157; BF16 N = 8 128 / 104, 11 181 / 168; on the fly N = 6 199 / 173, 8 237 /
 // 150, 11 257 / 242; FP64 N = 15 1327 / 1270.
 template <int NP, typename T, int EB_, bool STAGE, bool BOXM, typename TG, bool DOT>
-__global__ void __launch_bounds__(ApplyCfg<NP, EB_>::NT, apply_min_blocks<T, TG, !BOXM && !DOT>(NP, EB_))
+__global__ void __launch_bounds__(ApplyCfg<NP, EB_>::NT, apply_min_blocks<T, TG, BOXM, DOT>(NP, EB_))
     k_apply(const ApplyParams<T, NP> P) {
   using C = ApplyCfg<NP, EB_>;
   constexpr int N = NP - 1, NP2 = C::NP2, NP3 = C::NP3, EB = C::EB, NT = C::NT, RS = C::RS, PS = C::PS,
                 BUF = C::BUF, GS = factor_stride<NP, TG>();
   extern __shared__ __align__(128) unsigned char smem_raw[];
   constexpr size_t RED_OFF = apply_red_off<NP, T, EB_, STAGE, TG>();
-  constexpr bool PK = BOXM && apply_packed<T, TG>(NP);
+  constexpr bool PK = (BOXM || DOT) && apply_packed<T, TG>(NP);
   static_assert(RED_OFF % 16 == 0 && ((STAGE ? EB * GS : 0) * sizeof(TG)) % 16 == 0, "shared-memory alignment");
   TG *sG = reinterpret_cast<TG *>(smem_raw);  // TMA destination: 16-byte aligned at offset 0
   T *sbuf = reinterpret_cast<T *>(smem_raw + (STAGE ? EB * GS * sizeof(TG) : 0));
@@ -420,7 +424,7 @@ __global__ void __launch_bounds__(ApplyCfg<NP, EB_>::NT, apply_min_blocks<T, TG,
       if (__syncthreads_and(skip)) return;  // every element of this block is finished
     }
   }
-  constexpr bool PREF = BOXM && apply_prefetch<T, TG, STAGE>(NP);
+  constexpr bool PREF = (BOXM || DOT) && apply_prefetch<T, TG, STAGE>(NP);
   TG gpre[PREF ? 6 * NP : 1];
   if constexpr (PREF) {
     const TG *Ge = c_Gf + (active ? el : 0) * P.gs + t2;
@@ -648,9 +652,9 @@ __global__ void __launch_bounds__(ApplyCfg<NP, EB_>::NT, apply_min_blocks<T, TG,
         atomicAdd(P.y + g, yk);
     }
   };
-  // Optional arrays are tested through their own pointers, here and for kappa above: a pointer that was
-  // offset first ("q ? q + i : nullptr") and then tested was dereferenced with q null in the FP64 form
-  // of this kernel, where a build of the same source for the host is clean.
+  // Optional arrays are tested through their own pointers, here and for kappa above.  Builds of this kernel that
+  // offset them first ("q ? q + i : nullptr") and tested the result were among those that faulted; the pattern is
+  // valid C++ and ran without a fault in others, so it is a suspicion only, and it is avoided.
   if (DOT && P.partials) {
     // p^T A p and the CG step length: one warp adds the block's terms and publishes them before its
     // scatter, so that its fences have no writes to wait for and the other warps do not wait at all
@@ -787,7 +791,10 @@ __host__ __device__ constexpr int apply_auto_variant(int NP, bool general) {
 //
 // Registers: small orders ask for their factors with u, beside the gather and the gradients (an element
 // alone on an SM waits for them otherwise); from N = 9 those registers are worth more as resident blocks
-// (N = 9 at 8e6 nodes: 6.8 with the factors held, 8.2 without, 8.8 at three blocks per SM).
+// (N = 9 at 8e6 nodes: 6.8 with the factors held, 8.2 without, 8.8 at three blocks per SM).  At two blocks per SM
+// N = 11 has 72 registers and no spill; N = 12, 13 and 14 have 64, 48 and 40 and spill (160, 330 and 550 bytes a
+// thread), and are the faster for it at size: two / one block per SM (94, 95 and 80 registers), 15^3, 14^3 and 13^3
+// elements, 941 / 1076, 1051 / 1169, 1065 / 1162 us; 5^3, 5^3 and 4^3 49.1 / 46.8, 62.8 / 62.8, 77.7 / 77.7.
 constexpr int cols_min_blocks(int NP) { return NP <= 9 ? 1 : NP == 10 ? 3 : 2; }
 
 // Orders and sizes it is for (k_apply / this kernel): N = 5 to 9, 11 and 12 at every size (N = 5: 64 elements
@@ -795,9 +802,9 @@ constexpr int cols_min_blocks(int NP) { return NP <= 9 ? 1 : NP == 10 ? 3 : 2; }
 // 48.4); N = 3 and 4, whose k_apply blocks hold 8 and 5 elements, up to four and three elements per SM (N = 3:
 // 729 elements 9.9 / 9.1, 1000 10.0 / 10.8; N = 4: 343 11.7 / 9.4, 512 11.7 / 11.1, 729 11.7 / 13.0); N = 13 and 14
 // from two elements per SM (N = 13: 125 elements 62.7 / 64.7, 8e6 nodes 6.0 / 7.1 GDOF/s).  Not N = 10 (125
-// elements 28.3 / 30.1, 343 74 / 81), and not N = 15, which spills at the 80 registers that are left.
+// elements 28.3 / 30.1, 343 74 / 81), and not N = 15 (768 threads, 80 registers at one block per SM).
 constexpr bool apply_cols(int NP, int64_t E) {
-  return NP == 4 ? E <= 4 * 152 : NP == 5 ? E <= 3 * 152 : NP == 14 || NP == 15 ? E > 2 * 152 : NP >= 6 && NP <= 13 && NP != 11;
+  return NP == 4 ? E <= 4 * SEM_SMS : NP == 5 ? E <= 3 * SEM_SMS : NP == 14 || NP == 15 ? E > 2 * SEM_SMS : NP >= 6 && NP <= 13 && NP != 11;
 }
 
 template <int NP, bool BOXM>

@@ -244,7 +244,7 @@ int tiles(const GemmArgs &g) {
 
 // The 64 x 64 tile from one tile per SM (152) on, the split 32 x 16 tile below: with fewer large
 // tiles than SMs the rest of the chip idles.
-inline bool use_large(int large_tiles) { return large_tiles >= 152; }
+inline bool use_large(int large_tiles) { return large_tiles >= SEM_SMS; }
 
 template <bool TA, bool TB, int EP>
 sem_status gemm(const GemmArgs &g, cudaStream_t s) {

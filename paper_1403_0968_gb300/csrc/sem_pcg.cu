@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(VT) k_cg_init(int64_t G, const double *b, doub
 // Vectors that a kernel only reads, but the ones before it write, are not __restrict__: as dependent launches
 // these kernels begin before the writer has ended, and the read-only load path is for data that nothing
 // writes while the kernel lives.
-constexpr int UT = 512, UBLOCKS = 152 * 2;
+constexpr int UT = 512, UBLOCKS = SEM_SMS * 2;
 
 template <typename T>
 struct alignas(16) Vec16 {
@@ -448,7 +448,7 @@ sem_status fcg_block(sem_handle *h, int prec64, int count, double *x, cudaStream
     k_fcg_dots<<<vgrid(G), VT, 0, st>>>(G, h->z64, h->r64, h->Ap64, h->scal, h->partials, 0);
     // the fallback pair does work only after a rejected correction (rare): one block per SM of a
     // GB300 (152), so that the launches that find nothing to do cost little
-    const unsigned fb = std::min(vgrid(G), 152u);
+    const unsigned fb = std::min(vgrid(G), (unsigned)SEM_SMS);
     k_jacobi_z<<<fb, VT, 0, st>>>(G, h->r64, h->dinv64, h->z64, h->scal);
     k_fcg_dots<<<fb, VT, 0, st>>>(G, h->z64, h->r64, h->Ap64, h->scal, h->partials, 1);
     k_fcg_direction<<<vgrid(G), VT, 0, st>>>(G, h->p64, h->z64, h->Ap64, h->scal);
