@@ -600,7 +600,7 @@ __host__ __device__ constexpr DgRule dg_rule(int N) {
            : N == 5 ? DgRule{26, 1, 0, 1}
            : N == 6 ? DgRule{40, 2, 0, 2}
            : N == 7 ? DgRule{50, 2, 0, 2}
-                    : DgRule{25, 2, 0, 2};
+                    : DgRule{27, 2, 0, 2};
   return N == 1   ? DgRule{0, 4, 50, 0}
          : N == 2 ? DgRule{0, 0, 0, 0}
          : N == 3 ? DgRule{145, 1, 0, 1}
